@@ -5,9 +5,9 @@
 // Per step, in stream order:
 //   grad_sqnorm_kernel      global ||G||^2 for clipping (shared with the
 //                           elementwise path), when clipping is on
-//   muon_momentum_kernel    M <- mu M + (1 - mu) G^, and per-chunk partial
-//                           sums of M^2 (fixed chunks: deterministic)
-//   muon_norm_kernel        ||M||_F per matrix from its partials, in order
+//   muon_momentum_kernel    M <- mu M + (1 - mu) G^, per-chunk partial sums of
+//                           M^2 (fixed chunks: deterministic) and, by the last
+//                           CTA of each matrix, 1 / (||M||_F + eps)
 //   muon_normalize_kernel   X_0 = bf16(M / (||M||_F + eps)) into the padded
 //                           workspace, in the wide orientation (64 x 64 tiles
 //                           through shared memory)
@@ -40,12 +40,14 @@
 
 #include "dpo_device.cuh"
 #include "dpo_gemm.cuh"
+#include "dpo_reduce.cuh"
 
 namespace dpo {
 namespace muon {
 
 constexpr int kThreads = 256;
-constexpr int64_t kChunk = (int64_t)kThreads * kPacket * 16;  // elements per momentum CTA
+constexpr int64_t kRound = (int64_t)kThreads * kPacket;   // elements of one CTA round (2048)
+constexpr int64_t kMaxChunk = 16 * kRound;                // elements per CTA, at most
 constexpr int kPad = 256;                                       // workspace padding
 
 struct DevMat {
@@ -62,12 +64,69 @@ struct DevMat {
     int sync;                 // DPO_SYNC: trained synchronously (no stash, no history)
 };
 
+// The momentum, update and prediction passes are flat over all matrices:
+// matrix i owns chunks [begin[i], begin[i + 1]) of `elems` elements each, one
+// CTA per chunk. One CTA row per matrix, as wide as the largest matrix, left
+// a set of small matrices on a dozen CTAs (two 256 x 768 matrices: 7.9 us of
+// momentum, 11.7 us of update) and launched mostly empty CTAs where sizes
+// differ.
+struct Chunks {
+    const int *begin;         // n + 1 prefix offsets
+    int n;
+    int elems;                // elements per chunk, a multiple of kRound
+};
+
+// The last matrix i with begin[i] <= c, by every warp at once: the lanes'
+// loads are independent, so the search costs one load latency per 32 matrices
+// (a binary search: one per bisection).
+__device__ __forceinline__ int find_mat(const int *begin, int n, int c)
+{
+    const int lane = threadIdx.x & 31;
+    int cnt = 0;
+    for (int i = 0; i < n; i += 32)
+        cnt += __popc(__ballot_sync(0xFFFFFFFFu, i + lane < n && __ldg(begin + i + lane) <= c));
+    return cnt - 1;
+}
+
+// Row and column of element e of a matrix with `cols` columns. The 64-bit
+// division is a subroutine of some 70 instructions; most matrices fit 32 bits.
+__device__ __forceinline__ void row_col(int64_t e, int64_t cols, bool small, int64_t &i, int64_t &j)
+{
+    i = small ? (int64_t)((uint32_t)e / (uint32_t)cols) : e / cols;
+    j = e - i * cols;
+}
+
+// Eight consecutive elements e.. of the Newton-Schulz output (row-major, pitch
+// o_ld): one 16-byte load where rows are whole packets, else element by
+// element, passing to the next row where a row ends inside the packet.
+__device__ __forceinline__ void load_o8(const DevMat &d, int64_t e, bool small, float (&o)[8])
+{
+    int64_t i, j;
+    row_col(e, d.cols, small, i, j);
+    if (d.cols % kPacket == 0) {
+        ld8(d.o + i * d.o_ld + j, o);
+        return;
+    }
+    const __nv_bfloat16 *row = d.o + i * d.o_ld;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        o[k] = __bfloat162float(row[j]);
+        if (++j == d.cols) {   // the packet ends inside the matrix, so a next row exists
+            j = 0;             // whenever an element of it is read
+            row += d.o_ld;
+        }
+    }
+}
+
 struct MomArgs {
     const DevMat *mats;
+    Chunks ch;
     const float *clip;        // device clip coefficient, or nullptr
     float mu, omm;
-    double *partials;         // [n_mats][chunks]
-    int chunks;
+    double *partials;         // one per chunk
+    unsigned int *tickets;    // per matrix: chunks done, 0 between launches
+    float eps;
+    float *inv_norm;          // per matrix: 1 / (||M||_F + eps)
     int predict;              // M' = mu M + (1 - mu) G^ into the history buffer of each
                               // delayed matrix; M keeps its value
 };
@@ -76,16 +135,19 @@ template <class GT>
 __global__ void __launch_bounds__(kThreads) muon_momentum_kernel(const MomArgs a)
 {
     __shared__ double red[kThreads / 32];
-    const DevMat &d = a.mats[blockIdx.y];
+    __shared__ bool last;
+    const int mi = find_mat(a.ch.begin, a.ch.n, (int)blockIdx.x);
+    const int c0 = __ldg(a.ch.begin + mi), c1 = __ldg(a.ch.begin + mi + 1);
+    const DevMat &d = a.mats[mi];
     // the prediction pass leaves a synchronous matrix (and its history) alone
     const bool skip = a.predict && (d.sync || d.ef == nullptr);
     const int64_t n = skip ? 0 : d.rows * d.cols;
     float *out = a.predict ? d.ef : d.mom;
-    const int64_t lo = (int64_t)blockIdx.x * kChunk;
+    const int64_t lo = (int64_t)((int)blockIdx.x - c0) * a.ch.elems;
     float sum = 0.0f, comp = 0.0f;
     if (lo < n) {
         const float clip = a.clip != nullptr ? __ldg(a.clip) : 1.0f;
-        const int64_t hi = lo + kChunk < n ? lo + kChunk : n;
+        const int64_t hi = lo + a.ch.elems < n ? lo + a.ch.elems : n;
         const GT *grad = static_cast<const GT *>(d.grad);
         for (int64_t e = lo + (int64_t)threadIdx.x * kPacket; e < hi; e += (int64_t)kThreads * kPacket) {
             if (e + kPacket <= hi) {
@@ -117,38 +179,29 @@ __global__ void __launch_bounds__(kThreads) muon_momentum_kernel(const MomArgs a
             }
         }
     }
-    double x = (double)sum - (double)comp;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1)
-        x += __shfl_down_sync(0xFFFFFFFFu, x, off);
-    if ((threadIdx.x & 31) == 0)
-        red[threadIdx.x >> 5] = x;
-    __syncthreads();
+    // The last CTA of the matrix to arrive adds its chunks' partials in a fixed
+    // order (strided over the threads, then the block's fixed tree), so the norm
+    // does not depend on arrival order. A kernel of its own for this took 2.5 us
+    // (two small matrices) to 9.5 us (a 7B layer's 1376 partials per matrix on
+    // one warp each) and a launch.
+    const double cta = block_sum<kThreads>((double)sum - (double)comp, red);
     if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < kThreads / 32; ++w)
-            s += red[w];
-        a.partials[(int64_t)blockIdx.y * a.chunks + blockIdx.x] = s;
+        a.partials[blockIdx.x] = cta;
+        __threadfence();
+        last = atomicAdd(&a.tickets[mi], 1u) == (unsigned)(c1 - c0 - 1);
     }
-}
-
-// 1 / (||M||_F + eps) per matrix: one warp per matrix sums its partials in a
-// fixed order (lane-strided, then a fixed shuffle tree).
-__global__ void muon_norm_kernel(const double *partials, int chunks, int n_mats, float eps,
-                                 float *inv_norm)
-{
-    const int mat = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (mat >= n_mats)
+    __syncthreads();
+    if (!last)
         return;
-    double s = 0.0;
-    for (int c = lane; c < chunks; c += 32)
-        s += partials[(int64_t)mat * chunks + c];
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1)
-        s += __shfl_down_sync(0xFFFFFFFFu, s, off);
-    if (lane == 0)
-        inv_norm[mat] = (float)(1.0 / (sqrt(s) + (double)eps));
+    __threadfence();
+    double acc = 0.0;
+    for (int c = c0 + (int)threadIdx.x; c < c1; c += kThreads)
+        acc += __ldcg(a.partials + c);
+    const double total = block_sum<kThreads>(acc, red);
+    if (threadIdx.x == 0) {
+        a.inv_norm[mi] = (float)(1.0 / (sqrt(total) + (double)a.eps));
+        a.tickets[mi] = 0u;   // ready for the next launch
+    }
 }
 
 struct NormArgsM {
@@ -241,7 +294,7 @@ struct MuonCounters {
 
 struct ApplyArgs {
     const DevMat *mats;
-    int chunks;
+    Chunks ch;
     float lr, lr_wd, lam;
     int ef_now, hist, delayed;
     int sapipe;               // SAPipe-WP: stash := x_t - U_prev, standard rule
@@ -270,28 +323,26 @@ template <int SK>
 __global__ void __launch_bounds__(kThreads) muon_apply_kernel(const ApplyArgs a)
 {
     using ST = typename StashT<SK>::T;
-    const DevMat &d = a.mats[blockIdx.y];
+    const int mi = find_mat(a.ch.begin, a.ch.n, (int)blockIdx.x);
+    const DevMat &d = a.mats[mi];
     const int64_t n = d.rows * d.cols;
-    const int64_t lo = (int64_t)blockIdx.x * kChunk;
-    if (lo >= n)
-        return;
-    const int64_t hi = lo + kChunk < n ? lo + kChunk : n;
+    const int64_t lo = (int64_t)((int)blockIdx.x - __ldg(a.ch.begin + mi)) * a.ch.elems;
+    const int64_t hi = lo + a.ch.elems < n ? lo + a.ch.elems : n;
     const ApplyScalars sc = a.dev != nullptr ? *a.dev : ApplyScalars{a.lr, a.lr_wd, a.ef_now};
     const float lr_r = sc.lr * d.r_scale, lr_wd = sc.lr_wd * d.wd_lr_scale;
     ST *stash = static_cast<ST *>(d.stash);
     __nv_bfloat16 *param = static_cast<__nv_bfloat16 *>(d.param);
-    const bool vec_o = (d.cols % kPacket) == 0;
+    const bool small = n <= (int64_t)UINT32_MAX;
     // a DPO_SYNC matrix takes the standard update with no stash and no history
     const bool dly = a.delayed && !d.sync;
     const bool hist = a.hist && dly, ef_now = sc.ef_now && dly;
     const bool sapipe = a.sapipe && hist;
     const bool write_hist = hist && !a.keep_hist;
     for (int64_t e = lo + (int64_t)threadIdx.x * kPacket; e < hi; e += (int64_t)kThreads * kPacket) {
-        if (e + kPacket <= hi && vec_o) {
-            const int64_t i = e / d.cols, j = e - i * d.cols;
+        if (e + kPacket <= hi) {
             float x[8], o[8], up[8], u[8];
             ld8(d.master + e, x);
-            ld8(d.o + i * d.o_ld + j, o);
+            load_o8(d, e, small, o);
             if (ef_now || sapipe)
                 ld8(d.ef + e, up);
             if (SK != kStashNone && dly) {
@@ -316,8 +367,7 @@ __global__ void __launch_bounds__(kThreads) muon_apply_kernel(const ApplyArgs a)
             if (param != nullptr)
                 st8(param + e, x);
         } else {
-            const int64_t top = e + kPacket < hi ? e + kPacket : hi;
-            for (int64_t q = e; q < top; ++q) {
+            for (int64_t q = e; q < hi; ++q) {   // the matrix's last, partial packet
                 const int64_t i = q / d.cols, j = q - i * d.cols;
                 float x = d.master[q];
                 const float o = __bfloat162float(d.o[i * d.o_ld + j]);
@@ -340,30 +390,27 @@ __global__ void __launch_bounds__(kThreads) muon_apply_kernel(const ApplyArgs a)
 // Newton-Schulz output of M' and X_{t+1} the master the real update left.
 __global__ void __launch_bounds__(kThreads) muon_predict_kernel(const ApplyArgs a)
 {
-    const DevMat &d = a.mats[blockIdx.y];
+    const int mi = find_mat(a.ch.begin, a.ch.n, (int)blockIdx.x);
+    const DevMat &d = a.mats[mi];
     if (d.sync || d.ef == nullptr)
         return;
     const int64_t n = d.rows * d.cols;
-    const int64_t lo = (int64_t)blockIdx.x * kChunk;
-    if (lo >= n)
-        return;
-    const int64_t hi = lo + kChunk < n ? lo + kChunk : n;
+    const int64_t lo = (int64_t)((int)blockIdx.x - __ldg(a.ch.begin + mi)) * a.ch.elems;
+    const int64_t hi = lo + a.ch.elems < n ? lo + a.ch.elems : n;
     const ApplyScalars sc = a.dev != nullptr ? *a.dev : ApplyScalars{a.lr, a.lr_wd, a.ef_now};
     const float lr_r = sc.lr * d.r_scale, lr_wd = sc.lr_wd * d.wd_lr_scale;
-    const bool vec_o = (d.cols % kPacket) == 0;
+    const bool small = n <= (int64_t)UINT32_MAX;
     for (int64_t e = lo + (int64_t)threadIdx.x * kPacket; e < hi; e += (int64_t)kThreads * kPacket) {
-        if (e + kPacket <= hi && vec_o) {
-            const int64_t i = e / d.cols, j = e - i * d.cols;
+        if (e + kPacket <= hi) {
             float x[8], o[8], u[8];
             ld8(d.master + e, x);
-            ld8(d.o + i * d.o_ld + j, o);
+            load_o8(d, e, small, o);
 #pragma unroll
             for (int k = 0; k < 8; ++k)
                 u[k] = fmaf(lr_r, o[k], lr_wd * x[k]);
             st8(d.ef + e, u);
         } else {
-            const int64_t top = e + kPacket < hi ? e + kPacket : hi;
-            for (int64_t q = e; q < top; ++q) {
+            for (int64_t q = e; q < hi; ++q) {
                 const int64_t i = q / d.cols, j = q - i * d.cols;
                 d.ef[q] = fmaf(lr_r, __bfloat162float(d.o[i * d.o_ld + j]), lr_wd * d.master[q]);
             }
@@ -407,7 +454,6 @@ namespace {
 using dpo::muon::DevMat;
 using dpo::muon::kPad;
 using dpo::muon::kThreads;
-using dpo::muon::kChunk;
 
 thread_local std::string g_muon_init_err;
 
@@ -502,7 +548,8 @@ struct dpo_muon_ctx {
     std::vector<dpo_matrix> mats;
     std::vector<DevMat> host_mats;
     std::vector<Group> groups;
-    int chunks = 0;
+    int n_chunks = 0;         // CTAs of the momentum, update and prediction passes
+    int chunk_elems = 0;
     int64_t total_elems = 0;
     int64_t ws_bytes = 0;
     double flops = 0.0;
@@ -510,7 +557,9 @@ struct dpo_muon_ctx {
     void *dev_block = nullptr;
     void *ws = nullptr;
     DevMat *d_mats = nullptr;
+    int *d_chunk_begin = nullptr;
     double *d_partials = nullptr;
+    unsigned int *d_tickets = nullptr;
     float *d_inv_norm = nullptr;
     unsigned int *d_err = nullptr;
     // gradient norm for clipping (the elementwise path's kernel and table)
@@ -658,12 +707,10 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
 
     // Group the matrices by their wide orientation r x w (r <= w).
     std::map<std::pair<int64_t, int64_t>, int> gidx;
-    int64_t max_n = 0;
     for (int i = 0; i < n; ++i) {
         const dpo_matrix &m = mats[i];
         const int64_t ne = m.rows * m.cols;
         c->total_elems += ne;
-        max_n = std::max(max_n, ne);
         if (ne == 0)
             continue;
         const int64_t r = std::min(m.rows, m.cols), w = std::max(m.rows, m.cols);
@@ -683,7 +730,27 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
         c->flops += (double)hp->ns_steps * ((double)r * (r + 1) * w + (double)r * (r + 1) * r +
                                             2.0 * (double)r * r * w);
     }
-    c->chunks = (int)std::max<int64_t>(1, (max_n + kChunk - 1) / kChunk);
+    // Chunks of the flat passes: about 16 CTAs per SM, so a set of a few
+    // million elements still covers the SMs several times over, and at most
+    // kMaxChunk elements each, where a CTA's fixed cost no longer shows.
+    const int64_t want = c->total_elems / (16 * (int64_t)std::max(1, c->sms));
+    int64_t ce = std::max<int64_t>(
+        dpo::muon::kRound,
+        std::min<int64_t>(dpo::muon::kMaxChunk,
+                          (want + dpo::muon::kRound - 1) / dpo::muon::kRound * dpo::muon::kRound));
+    std::vector<int> chunk_begin(n + 1, 0);
+    int64_t n_chunks = 0;
+    for (int i = 0; i < n; ++i) {
+        chunk_begin[i] = (int)n_chunks;
+        n_chunks += (mats[i].rows * mats[i].cols + ce - 1) / ce;
+    }
+    if (n_chunks > INT32_MAX) {   // 2^31 chunks of kMaxChunk: 281 TB of fp32
+        free_ctx(c);
+        return mfail(nullptr, DPO_EINVAL, "too many elements");
+    }
+    chunk_begin[n] = (int)n_chunks;
+    c->n_chunks = (int)n_chunks;
+    c->chunk_elems = (int)ce;
 
     // Workspace: per group X twice, X^T (the output of tall matrices), A, B (bf16).
     int64_t ws = 0;
@@ -723,7 +790,11 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
         off += al((int64_t)sizeof(int) * (int64_t)g.mats.size());
     }
     const int64_t o_part = off;
-    off += al((int64_t)sizeof(double) * std::max(1, n) * c->chunks);
+    off += al((int64_t)sizeof(double) * std::max(1, c->n_chunks));
+    const int64_t o_cbeg = off;
+    off += al((int64_t)sizeof(int) * (n + 1));
+    const int64_t o_tick = off;
+    off += al((int64_t)sizeof(unsigned int) * std::max(1, n));
     const int64_t o_inv = off;
     off += al((int64_t)sizeof(float) * std::max(1, n));
     const int64_t o_err = off;
@@ -757,6 +828,8 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
     char *blk = static_cast<char *>(c->dev_block);
     c->d_mats = reinterpret_cast<DevMat *>(blk + o_mats);
     c->d_partials = reinterpret_cast<double *>(blk + o_part);
+    c->d_chunk_begin = reinterpret_cast<int *>(blk + o_cbeg);
+    c->d_tickets = reinterpret_cast<unsigned int *>(blk + o_tick);
     c->d_inv_norm = reinterpret_cast<float *>(blk + o_inv);
     c->d_err = reinterpret_cast<unsigned int *>(blk + o_err);
     c->d_norm_table = reinterpret_cast<dpo::DevTensor *>(blk + o_ntab);
@@ -854,10 +927,13 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
         MUON_COPY(g.d_mats, g.mats.data(), sizeof(int) * g.mats.size());
     MUON_COPY(c->d_norm_table, ntab.data(), sizeof(dpo::DevTensor) * n);
     MUON_COPY(c->d_pkt_begin, pkt_begin.data(), sizeof(int64_t) * (n + 1));
+    MUON_COPY(c->d_chunk_begin, chunk_begin.data(), sizeof(int) * (n + 1));
 #undef MUON_COPY
     e = cudaMemsetAsync(c->d_err, 0, sizeof(unsigned int), s);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(c->d_norm_scalars, 0, sizeof(dpo::NormScalars), s);
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(c->d_tickets, 0, sizeof(unsigned int) * std::max(1, n), s);
     if (e == cudaSuccess && ws > 0)
         e = cudaMemsetAsync(c->ws, 0, (size_t)ws, s);   // zero padding stays zero
     if (e != cudaSuccess) {
@@ -982,13 +1058,16 @@ int orthogonalize(dpo_muon_ctx *c, cudaStream_t s, bool predict)
     // momentum and its Frobenius norms
     dpo::muon::MomArgs ma{};
     ma.mats = c->d_mats;
+    ma.ch = dpo::muon::Chunks{c->d_chunk_begin, c->n, c->chunk_elems};
     ma.clip = c->hp.max_grad_norm > 0.0f ? &c->d_norm_scalars->clip : nullptr;
     ma.mu = c->hp.momentum;
     ma.omm = (float)(1.0 - (double)c->hp.momentum);
     ma.partials = c->d_partials;
-    ma.chunks = c->chunks;
+    ma.tickets = c->d_tickets;
+    ma.eps = c->hp.ns_eps;
+    ma.inv_norm = c->d_inv_norm;
     ma.predict = predict ? 1 : 0;
-    const dim3 mgrid((unsigned)c->chunks, (unsigned)c->n);
+    const unsigned mgrid = (unsigned)c->n_chunks;
     if (c->grad_dt == DPO_BF16)
         dpo::muon::muon_momentum_kernel<__nv_bfloat16><<<mgrid, kThreads, 0, s>>>(ma);
     else
@@ -996,11 +1075,6 @@ int orthogonalize(dpo_muon_ctx *c, cudaStream_t s, bool predict)
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return mcuda(c, e, "momentum launch");
-    dpo::muon::muon_norm_kernel<<<(c->n + 7) / 8, 256, 0, s>>>(c->d_partials, c->chunks, c->n,
-                                                               c->hp.ns_eps, c->d_inv_norm);
-    if ((e = cudaGetLastError()) != cudaSuccess)
-        return mcuda(c, e, "norm launch");
-
     for (Group &g : c->groups) {
         const int64_t nb = (int64_t)g.mats.size();
         dpo::muon::NormArgsM na{c->d_mats, g.d_mats, c->d_inv_norm, g.x[0],
@@ -1137,13 +1211,13 @@ extern "C" int dpo_muon_step(dpo_muon_ctx *c, float lr, void *stream)
     if (rc != DPO_OK)
         return rc;
     cudaError_t e;
-    const dim3 mgrid((unsigned)c->chunks, (unsigned)c->n);
+    const unsigned mgrid = (unsigned)c->n_chunks;
 
     // update, stash, history, weights
     const int64_t t = k - c->phase_k0;   // Alg. 1 iteration within the delayed phase
     dpo::muon::ApplyArgs aa{};
     aa.mats = c->d_mats;
-    aa.chunks = c->chunks;
+    aa.ch = dpo::muon::Chunks{c->d_chunk_begin, c->n, c->chunk_elems};
     aa.lr = lr;
     aa.lr_wd = (float)((double)lr * (double)c->hp.weight_decay);
     aa.delayed = c->hp.delay == 1;

@@ -1,0 +1,39 @@
+"""The flat work lists of delayed Muon's element-wise passes against the
+oracle (Alg. 2), at the sizes where the split can go wrong: matrices one
+element short of, at and past one round of a CTA (2048), widths that are no
+whole packets (a packet of the update then spans two or more rows), a last
+partial packet, empty matrices at either end, and more matrices than one warp
+searches at a time (32)."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from parity_util import TOL_ONE_STEP, TOL_RUN, rel_err
+from test_muon_parity import F, Pair, _flat, close_with_flips
+
+pytestmark = pytest.mark.gpu
+
+EDGES = [(0, 4), (1, 2047), (1, 2048), (1, 2049), (2049, 1), (683, 3), (7, 293), (64, 33), (5, 0)]
+MANY = [(1 + i % 5, (3 * i) % 23) for i in range(70)] + [(9, 515), (0, 0)]
+
+
+@pytest.mark.parametrize("shapes", [EDGES, MANY], ids=["edges", "many"])
+@pytest.mark.parametrize("correction", [0, 2])
+def test_flat_chunks_match_the_oracle(cuda_device, shapes, correction):
+    """Three calls, no Newton-Schulz steps, so O is M / ||M||_F in bf16 and
+    the weights, momentum and history are held element by element; an O that
+    rounds the other way (an inverse norm one ulp off) moves U by at most
+    lr r 2^-8."""
+    p = Pair(shapes, cuda_device, ns_steps=0, ef=True, sdt=F, correction=correction)
+    du = p.lr * 0.2 * np.sqrt(max(max(s) for s in shapes)) * 2.0 ** -8
+    try:
+        for k in range(3):
+            p.step()
+            assert rel_err(p.cat(p.gpu.mom), _flat(p.ref.mom)) <= (TOL_ONE_STEP if k == 0
+                                                                   else TOL_RUN)
+            close_with_flips(p.cat(p.gpu.master), _flat(p.ref.x), TOL_RUN, (k + 1) * du, 1e-3)
+            close_with_flips(p.cat(p.gpu.ef), _flat(p.ref.u_prev), 1e-5, du, 2e-3)
+            close_with_flips(p.cat(p.gpu.stash), _flat(p.ref.stash), TOL_RUN, (k + 1) * du, 1e-3)
+    finally:
+        p.close()
