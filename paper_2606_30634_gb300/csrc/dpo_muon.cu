@@ -9,8 +9,7 @@
 //                           M^2 (fixed chunks: deterministic) and, by the last
 //                           CTA of each matrix, 1 / (||M||_F + eps)
 //   muon_normalize_kernel   X_0 = bf16(M / (||M||_F + eps)) into the padded
-//                           workspace, in the wide orientation (64 x 64 tiles
-//                           through shared memory)
+//                           workspace, in the wide orientation
 //   ns_gemm_kernel x 3 per Newton-Schulz step and matrix shape, batched over
 //                           every matrix of that shape (dpo_gemm.cuh):
 //                             A = X X^T;  B = c A A + b A;  X <- B X + a X
@@ -59,6 +58,8 @@ struct DevMat {
     int64_t rows, cols;
     const __nv_bfloat16 *o;   // Newton-Schulz output (workspace), row-major, pitch o_ld
     int64_t o_ld;
+    __nv_bfloat16 *x, *xt;    // workspace: X_0 (R x W) and X^T (W x R)
+    int64_t R, W;             // padded r <= w of the wide orientation
     float wd_lr_scale;        // 1 with DPO_WD_ON, else 0
     float r_scale;            // rms_scale sqrt(max(rows, cols)), or 1
     int sync;                 // DPO_SYNC: trained synchronously (no stash, no history)
@@ -204,78 +205,130 @@ __global__ void __launch_bounds__(kThreads) muon_momentum_kernel(const MomArgs a
     }
 }
 
-struct NormArgsM {
+// The normalisation works on tiles of kTile elements of X, one CTA each, over
+// all matrices in one launch (matrix i owns tiles [begin[i], begin[i + 1])):
+// kTileI x kTileJ of them where M is transposed, else kTile in a row.
+constexpr int kTileI = 64, kTileJ = 128, kTile = kTileI * kTileJ;
+
+struct NormalizeArgs {
     const DevMat *mats;
-    const int *group_mats;    // global matrix index of each batch entry
+    const int *tile_begin;    // n + 1 prefix offsets
+    int n;
     const float *inv_norm;
-    __nv_bfloat16 *x, *xt;    // X (R x W) and X^T (W x R, or nullptr) of batch entry 0
-    int64_t R, W;
-    int64_t r, w;
+    int write_xt;             // no Newton-Schulz steps: X_0^T is the output of tall matrices
     int predict;              // read M' from the history buffer (zeros for a
                               // synchronous matrix) instead of M
 };
 
-// One 64 x 64 tile of X (rows i over r, columns j over w) per CTA; padding
-// outside r x w is written as zero. M is read along its own rows (32-byte
-// fp32 vectors where the row pitch allows) and X written along its rows
-// (16-byte bf16 vectors), through a shared-memory tile that transposes the
-// tall matrices.
-__global__ void __launch_bounds__(kThreads) muon_normalize_kernel(const NormArgsM a)
+// Element (i, j) of the shared tile: rows of kTileJ floats whose 16-byte
+// groups are permuted by the row, so that 4 consecutive j at 8 rows i that are
+// 8 apart (a warp's transposing store) and 32 groups of one row (its load)
+// each take all 32 banks once.
+__device__ __forceinline__ int tile_at(int i, int j)
 {
-    __shared__ float tile[64][65];
-    const int bz = blockIdx.z;
-    const int gm = a.group_mats[bz];
-    const DevMat &d = a.mats[gm];
-    const bool tall = d.rows > d.cols;
-    const float s = a.inv_norm[gm];
+    return i * kTileJ + (((j >> 2) ^ ((i ^ (i >> 3)) & 7)) << 2) + (j & 3);
+}
+
+// X_0 = bf16(M / (||M||_F + eps)) in the wide orientation, zero outside r x w.
+// HBM-bound: 4 bytes in, 2 out per element. A wide matrix of whole packets has
+// X's rows where M has them and is streamed through registers, four packets
+// in flight per thread; a tall one is transposed through shared memory, and so
+// are widths of no whole packets, whose rows start at any 4-byte address: they
+// are loaded element by element, consecutive lanes on consecutive elements.
+// GB300, against 64 x 64 tiles through padded shared memory for every matrix
+// and one launch per shape: a 7B layer 227 -> 205 us (5.9 TB/s), GPT-2's set
+// 97 -> 89 us, four 1B layers 258 -> 250 us, odd shapes 23 -> 20 us and four
+// launches fewer.
+__global__ void __launch_bounds__(kThreads) muon_normalize_kernel(const NormalizeArgs a)
+{
+    __shared__ __align__(16) float tile[kTile];
+    const int mi = find_mat(a.tile_begin, a.n, (int)blockIdx.x);
+    const DevMat &d = a.mats[mi];
+    const int t = (int)blockIdx.x - __ldg(a.tile_begin + mi);
+    const bool tall = d.rows > d.cols, packets = d.cols % kPacket == 0;
+    const float s = a.inv_norm[mi];
     const float *src = a.predict ? (d.sync ? nullptr : d.ef) : d.mom;
-    const int64_t i0 = (int64_t)blockIdx.y * 64, j0 = (int64_t)blockIdx.x * 64;
-    // tile origin in M: (mr0, mc0), 64 x 64, clipped to rows x cols
-    const int64_t mr0 = tall ? j0 : i0, mc0 = tall ? i0 : j0;
-    const bool vec = (d.cols % kPacket) == 0 && mr0 + 64 <= d.rows && mc0 + 64 <= d.cols;
+    constexpr int kVec = kTile / kPacket / kThreads;   // packets per thread
+    if (!tall && packets) {
+        const int64_t at = (int64_t)t * kTile;
+        const int64_t ib = at / d.W;
+        const uint32_t jb = (uint32_t)(at - ib * d.W), W = (uint32_t)d.W;
+        float x[kVec][8];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int v = (int)threadIdx.x + h * kThreads;   // 512 vectors of 8
-        const int row = v >> 3, c8 = (v & 7) * 8;         // within the tile, in M's layout
-        float x[8];
-        if (src == nullptr) {
+        for (int h = 0; h < kVec; ++h) {
+            const uint32_t q = jb + (threadIdx.x + h * kThreads) * kPacket;
+            const int64_t i = ib + q / W, j = q % W;
+            if (src != nullptr && i < d.rows && j < d.cols) {
+                ld8(src + i * d.cols + j, x[h]);
+            } else {
 #pragma unroll
-            for (int e = 0; e < 8; ++e)
-                x[e] = 0.0f;
-        } else if (vec) {
-            ld8(src + (mr0 + row) * d.cols + mc0 + c8, x);
-        } else {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int64_t mr = mr0 + row, mc = mc0 + c8 + e;
-                x[e] = (mr < d.rows && mc < d.cols) ? src[mr * d.cols + mc] : 0.0f;
+                for (int e = 0; e < 8; ++e)
+                    x[h][e] = 0.0f;
             }
         }
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            if (tall)
-                tile[c8 + e][row] = x[e] * s;   // X row = M column
-            else
-                tile[row][c8 + e] = x[e] * s;
+        for (int h = 0; h < kVec; ++h) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                x[h][e] *= s;
+            st8(d.x + at + (threadIdx.x + h * kThreads) * kPacket, x[h]);
+        }
+        return;
+    }
+    const int tiles_j = (int)(d.W / kTileJ);
+    const int64_t i0 = (int64_t)(t / tiles_j) * kTileI, j0 = (int64_t)(t % tiles_j) * kTileJ;
+    // the tile of M: rows mr0.., columns mc0..
+    const int64_t mr0 = tall ? j0 : i0, mc0 = tall ? i0 : j0;
+    if (packets) {   // tall: 8 packets per row of M
+        static_assert(kTileI / kPacket == 8, "packets per row of M");
+#pragma unroll
+        for (int h = 0; h < kVec; ++h) {
+            const int v = (int)threadIdx.x + h * kThreads;
+            const int row = v >> 3, c8 = (v & 7) * kPacket;
+            float x[8];
+            if (src != nullptr && mr0 + row < d.rows && mc0 + c8 < d.cols) {
+                ld8(src + (mr0 + row) * d.cols + mc0 + c8, x);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    x[e] = 0.0f;
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                tile[tile_at(c8 + e, row)] = x[e] * s;   // X row = M column
+        }
+    } else {
+        const int width = tall ? kTileI : kTileJ;
+#pragma unroll 8
+        for (int h = 0; h < kTile / kThreads; ++h) {
+            const int q = (int)threadIdx.x + h * kThreads;
+            const int row = q / width, col = q % width;
+            const float x = src != nullptr && mr0 + row < d.rows && mc0 + col < d.cols
+                                ? ld1(src + (mr0 + row) * d.cols + mc0 + col)
+                                : 0.0f;
+            tile[tall ? tile_at(col, row) : tile_at(row, col)] = x * s;
         }
     }
     __syncthreads();
-    __nv_bfloat16 *xb = a.x + (int64_t)bz * a.R * a.W;
-    __nv_bfloat16 *xt = a.xt != nullptr ? a.xt + (int64_t)bz * a.W * a.R : nullptr;
+    // one row of the tile per warp: 4 consecutive elements per lane
+    static_assert(kTileJ == 32 * 4, "one row of the tile per warp");
+    const int lane = (int)threadIdx.x & 31;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int v = (int)threadIdx.x + h * kThreads;
-        const int row = v >> 3, c8 = (v & 7) * 8;   // within the tile, in X's layout
-        float o[8];
+    for (int row = (int)threadIdx.x >> 5; row < kTileI; row += kThreads / 32) {
+        const float4 o = *reinterpret_cast<const float4 *>(tile + tile_at(row, lane * 4));
+        __stcs(reinterpret_cast<uint2 *>(d.x + (i0 + row) * d.W + j0 + lane * 4),
+               make_uint2(pack_bf16x2(o.x, o.y), pack_bf16x2(o.z, o.w)));
+    }
+    if (a.write_xt && tall) {
 #pragma unroll
-        for (int e = 0; e < 8; ++e)
-            o[e] = tile[row][c8 + e];
-        st8(xb + (i0 + row) * a.W + j0 + c8, o);
-        if (xt != nullptr) {   // X_0^T: the output of tall matrices when there are no steps
+        for (int h = 0; h < kVec; ++h) {
+            const int v = (int)threadIdx.x + h * kThreads;
+            const int row = v >> 3, c8 = (v & 7) * kPacket;   // row of X^T, its columns
+            float o[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e)
-                o[e] = tile[c8 + e][row];
-            st8(xt + (j0 + row) * a.R + i0 + c8, o);
+                o[e] = tile[tile_at(c8 + e, row)];
+            st8(d.xt + (j0 + row) * d.R + i0 + c8, o);
         }
     }
 }
@@ -514,7 +567,6 @@ int64_t pad_up(int64_t v) { return (v + kPad - 1) / kPad * kPad; }
 struct Group {
     int64_t r, w, R, W;
     std::vector<int> mats;
-    int *d_mats = nullptr;          // into the context's device block
     bool has_tall = false;
     // X ping-pongs between x[0] and x[1]: every tile of X <- B X + a X reads
     // all of the old X, so the new one goes to the other buffer.
@@ -550,6 +602,7 @@ struct dpo_muon_ctx {
     std::vector<Group> groups;
     int n_chunks = 0;         // CTAs of the momentum, update and prediction passes
     int chunk_elems = 0;
+    int n_tiles = 0;          // CTAs of the normalisation
     int64_t total_elems = 0;
     int64_t ws_bytes = 0;
     double flops = 0.0;
@@ -558,6 +611,7 @@ struct dpo_muon_ctx {
     void *ws = nullptr;
     DevMat *d_mats = nullptr;
     int *d_chunk_begin = nullptr;
+    int *d_tile_begin = nullptr;
     double *d_partials = nullptr;
     unsigned int *d_tickets = nullptr;
     float *d_inv_norm = nullptr;
@@ -738,19 +792,19 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
         dpo::muon::kRound,
         std::min<int64_t>(dpo::muon::kMaxChunk,
                           (want + dpo::muon::kRound - 1) / dpo::muon::kRound * dpo::muon::kRound));
-    std::vector<int> chunk_begin(n + 1, 0);
-    int64_t n_chunks = 0;
+    std::vector<int> chunk_begin(n + 1, 0), tile_begin(n + 1, 0);
+    int64_t n_chunks = 0, n_tiles = 0;   // below 2^31 for any set that fits the device
     for (int i = 0; i < n; ++i) {
-        chunk_begin[i] = (int)n_chunks;
-        n_chunks += (mats[i].rows * mats[i].cols + ce - 1) / ce;
+        const int64_t ne = mats[i].rows * mats[i].cols;
+        n_chunks += (ne + ce - 1) / ce;
+        chunk_begin[i + 1] = (int)n_chunks;
+        if (ne > 0)
+            n_tiles += pad_up(mats[i].rows) * pad_up(mats[i].cols) / dpo::muon::kTile;
+        tile_begin[i + 1] = (int)n_tiles;
     }
-    if (n_chunks > INT32_MAX) {   // 2^31 chunks of kMaxChunk: 281 TB of fp32
-        free_ctx(c);
-        return mfail(nullptr, DPO_EINVAL, "too many elements");
-    }
-    chunk_begin[n] = (int)n_chunks;
     c->n_chunks = (int)n_chunks;
     c->chunk_elems = (int)ce;
+    c->n_tiles = (int)n_tiles;
 
     // Workspace: per group X twice, X^T (the output of tall matrices), A, B (bf16).
     int64_t ws = 0;
@@ -778,20 +832,18 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
     c->norm_grid = (int)std::max<int64_t>(
         1, std::min<int64_t>(norm_groups, (int64_t)std::max(1, c->sms) * std::max(1, per_sm_norm)));
 
-    // Device block: mats | group index arrays | partials | inv_norm | err |
-    // norm table | pkt_begin | norm partials | norm scalars.
+    // Device block: mats | partials | chunk and tile prefixes | tickets |
+    // inv_norm | err | norm table | pkt_begin | norm partials | norm scalars |
+    // capturable counters and scalars.
     auto al = [](int64_t v) { return (v + 255) / 256 * 256; };
     int64_t off = 0;
     const int64_t o_mats = off;
     off += al((int64_t)sizeof(DevMat) * std::max(1, n));
-    std::vector<int64_t> o_groups;
-    for (Group &g : c->groups) {
-        o_groups.push_back(off);
-        off += al((int64_t)sizeof(int) * (int64_t)g.mats.size());
-    }
     const int64_t o_part = off;
     off += al((int64_t)sizeof(double) * std::max(1, c->n_chunks));
     const int64_t o_cbeg = off;
+    off += al((int64_t)sizeof(int) * (n + 1));
+    const int64_t o_tbeg = off;
     off += al((int64_t)sizeof(int) * (n + 1));
     const int64_t o_tick = off;
     off += al((int64_t)sizeof(unsigned int) * std::max(1, n));
@@ -829,6 +881,7 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
     c->d_mats = reinterpret_cast<DevMat *>(blk + o_mats);
     c->d_partials = reinterpret_cast<double *>(blk + o_part);
     c->d_chunk_begin = reinterpret_cast<int *>(blk + o_cbeg);
+    c->d_tile_begin = reinterpret_cast<int *>(blk + o_tbeg);
     c->d_tickets = reinterpret_cast<unsigned int *>(blk + o_tick);
     c->d_inv_norm = reinterpret_cast<float *>(blk + o_inv);
     c->d_err = reinterpret_cast<unsigned int *>(blk + o_err);
@@ -855,14 +908,15 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
         d.cols = m.cols;
         d.o = nullptr;
         d.o_ld = 0;
+        d.x = d.xt = nullptr;
+        d.R = d.W = 0;
         d.wd_lr_scale = (m.flags & DPO_WD_ON) ? 1.0f : 0.0f;
         d.r_scale = hp->rms_scale > 0.0f
                         ? (float)(hp->rms_scale * std::sqrt((double)std::max(m.rows, m.cols)))
                         : 1.0f;
         d.sync = (m.flags & DPO_SYNC) ? 1 : 0;
     }
-    for (size_t gi = 0; gi < c->groups.size(); ++gi) {
-        Group &g = c->groups[gi];
+    for (Group &g : c->groups) {
         const int64_t nb = (int64_t)g.mats.size();
         for (int q = 0; q < 2; ++q) {
             g.x[q] = reinterpret_cast<__nv_bfloat16 *>(wp);
@@ -874,7 +928,6 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
         wp += nb * g.R * g.R * 2;
         g.b = reinterpret_cast<__nv_bfloat16 *>(wp);
         wp += nb * g.R * g.R * 2;
-        g.d_mats = reinterpret_cast<int *>(blk + o_groups[gi]);
         const bool ok = make_map(&g.x128[0], g.x[0], g.R, g.W, nb, dpo::gemm::BM) &&
                         make_map(&g.x128[1], g.x[1], g.R, g.W, nb, dpo::gemm::BM) &&
                         make_map(&g.a128, g.a, g.R, g.R, nb, dpo::gemm::BM) &&
@@ -895,6 +948,10 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
         // when there are no steps, else by the last step).
         for (size_t bi = 0; bi < g.mats.size(); ++bi) {
             DevMat &d = c->host_mats[g.mats[bi]];
+            d.x = g.x[0] + (int64_t)bi * g.R * g.W;
+            d.xt = g.xt + (int64_t)bi * g.W * g.R;
+            d.R = g.R;
+            d.W = g.W;
             if (d.rows > d.cols) {
                 d.o = g.xt + (int64_t)bi * g.W * g.R;
                 d.o_ld = g.R;
@@ -923,11 +980,10 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
         }                                                                               \
     } while (0)
     MUON_COPY(c->d_mats, c->host_mats.data(), sizeof(DevMat) * n);
-    for (Group &g : c->groups)
-        MUON_COPY(g.d_mats, g.mats.data(), sizeof(int) * g.mats.size());
     MUON_COPY(c->d_norm_table, ntab.data(), sizeof(dpo::DevTensor) * n);
     MUON_COPY(c->d_pkt_begin, pkt_begin.data(), sizeof(int64_t) * (n + 1));
     MUON_COPY(c->d_chunk_begin, chunk_begin.data(), sizeof(int) * (n + 1));
+    MUON_COPY(c->d_tile_begin, tile_begin.data(), sizeof(int) * (n + 1));
 #undef MUON_COPY
     e = cudaMemsetAsync(c->d_err, 0, sizeof(unsigned int), s);
     if (e == cudaSuccess)
@@ -1075,16 +1131,11 @@ int orthogonalize(dpo_muon_ctx *c, cudaStream_t s, bool predict)
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return mcuda(c, e, "momentum launch");
-    for (Group &g : c->groups) {
-        const int64_t nb = (int64_t)g.mats.size();
-        dpo::muon::NormArgsM na{c->d_mats, g.d_mats, c->d_inv_norm, g.x[0],
-                                c->hp.ns_steps == 0 ? g.xt : nullptr, g.R, g.W, g.r, g.w,
-                                predict ? 1 : 0};
-        const dim3 ngrid((unsigned)(g.W / 64), (unsigned)(g.R / 64), (unsigned)nb);
-        dpo::muon::muon_normalize_kernel<<<ngrid, kThreads, 0, s>>>(na);
-        if ((e = cudaGetLastError()) != cudaSuccess)
-            return mcuda(c, e, "normalize launch");
-    }
+    const dpo::muon::NormalizeArgs na{c->d_mats, c->d_tile_begin, c->n, c->d_inv_norm,
+                                      c->hp.ns_steps == 0 ? 1 : 0, predict ? 1 : 0};
+    dpo::muon::muon_normalize_kernel<<<(unsigned)c->n_tiles, kThreads, 0, s>>>(na);
+    if ((e = cudaGetLastError()) != cudaSuccess)
+        return mcuda(c, e, "normalize launch");
     cudaEvent_t ev_end = nullptr;
     if (c->timing && c->hp.ns_steps > 0) {
         if (c->ev_used + 2 > c->ev_pool.size()) {
