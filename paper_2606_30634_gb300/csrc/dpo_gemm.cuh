@@ -40,6 +40,8 @@
 #include <cuda_bf16.h>
 #include <cstdint>
 
+#include "dpo_device.cuh"
+
 namespace dpo {
 namespace gemm {
 
@@ -389,6 +391,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
     const int n_tiles = L.n_tiles;
+    pdl_wait();
 
     if (warp == 0) {
         if (lane == 0) {

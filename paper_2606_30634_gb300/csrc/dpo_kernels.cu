@@ -41,6 +41,7 @@ __device__ void finish_clip(double total, double max_norm, NormScalars *out)
 
 __global__ void clip_from_sumsq_kernel(const double *sumsq, double max_norm, NormScalars *out)
 {
+    pdl_wait();
     finish_clip(*sumsq, max_norm, out);
 }
 
@@ -61,11 +62,16 @@ __global__ void __launch_bounds__(kNormThreads) grad_sqnorm_kernel(const NormArg
     const int64_t round = (int64_t)gridDim.x * kNormThreads * U;
     const int64_t first = (int64_t)blockIdx.x * kNormThreads * U + threadIdx.x;
     float sum = 0.0f, comp = 0.0f;
-    if (first < a.total_pkts) {
-        Cursor c;
+    Cursor c;
+    const GT *grad = nullptr;
+    int64_t numel = 0;
+    if (first < a.total_pkts) {   // the tables are constant: found before the wait
         c.seek(a.pkt_begin, a.n_tensors, first);
-        const GT *grad = static_cast<const GT *>(a.table[c.t].grad);
-        int64_t numel = a.table[c.t].numel;
+        grad = static_cast<const GT *>(a.table[c.t].grad);
+        numel = a.table[c.t].numel;
+    }
+    pdl_wait();
+    if (first < a.total_pkts) {
         for (int64_t base = first; base < a.total_pkts; base += round) {
             const GT *ptr[U];
             int cnt[U];   // elements of the packet: 8, 1..7 (a tensor's last), 0 (none)
@@ -238,17 +244,13 @@ cudaError_t launch_step(Optimizer opt, bool pb, StashKind sk, bool gb, Correctio
     StepFn f = pick_step_for(opt, pb, sk, gb, corr, dc, pp);
     if (f == nullptr)
         return cudaErrorInvalidValue;
-    f<<<grid, kStepThreads, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(f, dim3(grid), kStepThreads, 0, s, a);
 }
 
 cudaError_t launch_norm(bool gb, int grid, const NormArgs &a, cudaStream_t s)
 {
-    if (gb)
-        grad_sqnorm_kernel<1><<<grid, kNormThreads, 0, s>>>(a);
-    else
-        grad_sqnorm_kernel<0><<<grid, kNormThreads, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(gb ? grad_sqnorm_kernel<1> : grad_sqnorm_kernel<0>, dim3(grid), kNormThreads,
+                      0, s, a);
 }
 
 // NAdam's momentum schedule mu_i = beta1 (1 - 0.5 * 0.96^(i psi)).
@@ -261,6 +263,7 @@ __device__ double nadam_mu_dev(const ScalarConsts &k, int64_t i)
 __global__ void step_scalars_kernel(StepCounters *cnt, const float *lr_src, float lr_host,
                                     const ScalarConsts k, StepScalars *out)
 {
+    pdl_wait();
     const int64_t kk = cnt->k + 1;            // this call consumes the kk-th gradient
     const int64_t t = kk - cnt->phase_k0;     // Alg. 1 iteration within the delayed phase
     const float lr = lr_src != nullptr ? *lr_src : lr_host;
@@ -296,15 +299,13 @@ __global__ void step_scalars_kernel(StepCounters *cnt, const float *lr_src, floa
 cudaError_t launch_step_scalars(StepCounters *cnt, const float *lr_src, float lr,
                                 const ScalarConsts &k, StepScalars *out, cudaStream_t s)
 {
-    step_scalars_kernel<<<1, 1, 0, s>>>(cnt, lr_src, lr, k, out);
-    return cudaGetLastError();
+    return launch_pdl(step_scalars_kernel, dim3(1), 1, 0, s, cnt, lr_src, lr, k, out);
 }
 
 cudaError_t launch_clip_from_sumsq(const double *sumsq, double max_norm, NormScalars *out,
                                    cudaStream_t s)
 {
-    clip_from_sumsq_kernel<<<1, 1, 0, s>>>(sumsq, max_norm, out);
-    return cudaGetLastError();
+    return launch_pdl(clip_from_sumsq_kernel, dim3(1), 1, 0, s, sumsq, max_norm, out);
 }
 
 cudaError_t launch_stash(bool pb, StashKind sk, int grid, const StashArgs &a, cudaStream_t s)

@@ -140,6 +140,7 @@ __global__ void __launch_bounds__(kThreads) muon_momentum_kernel(const MomArgs a
     const int mi = find_mat(a.ch.begin, a.ch.n, (int)blockIdx.x);
     const int c0 = __ldg(a.ch.begin + mi), c1 = __ldg(a.ch.begin + mi + 1);
     const DevMat &d = a.mats[mi];
+    pdl_wait();
     // the prediction pass leaves a synchronous matrix (and its history) alone
     const bool skip = a.predict && (d.sync || d.ef == nullptr);
     const int64_t n = skip ? 0 : d.rows * d.cols;
@@ -246,6 +247,7 @@ __global__ void __launch_bounds__(kThreads) muon_normalize_kernel(const Normaliz
     const DevMat &d = a.mats[mi];
     const int t = (int)blockIdx.x - __ldg(a.tile_begin + mi);
     const bool tall = d.rows > d.cols, packets = d.cols % kPacket == 0;
+    pdl_wait();
     const float s = a.inv_norm[mi];
     const float *src = a.predict ? (d.sync ? nullptr : d.ef) : d.mom;
     constexpr int kVec = kTile / kPacket / kThreads;   // packets per thread
@@ -361,6 +363,7 @@ struct ApplyArgs {
 __global__ void muon_scalars_kernel(MuonCounters *cnt, const float *lr_src, float lr_host,
                                     double weight_decay, int ef_possible, ApplyScalars *out)
 {
+    pdl_wait();
     const int64_t k = cnt->k + 1;
     const int64_t t = k - cnt->phase_k0;
     const float lr = lr_src != nullptr ? *lr_src : lr_host;
@@ -381,6 +384,7 @@ __global__ void __launch_bounds__(kThreads) muon_apply_kernel(const ApplyArgs a)
     const int64_t n = d.rows * d.cols;
     const int64_t lo = (int64_t)((int)blockIdx.x - __ldg(a.ch.begin + mi)) * a.ch.elems;
     const int64_t hi = lo + a.ch.elems < n ? lo + a.ch.elems : n;
+    pdl_wait();
     const ApplyScalars sc = a.dev != nullptr ? *a.dev : ApplyScalars{a.lr, a.lr_wd, a.ef_now};
     const float lr_r = sc.lr * d.r_scale, lr_wd = sc.lr_wd * d.wd_lr_scale;
     ST *stash = static_cast<ST *>(d.stash);
@@ -445,6 +449,7 @@ __global__ void __launch_bounds__(kThreads) muon_predict_kernel(const ApplyArgs 
 {
     const int mi = find_mat(a.ch.begin, a.ch.n, (int)blockIdx.x);
     const DevMat &d = a.mats[mi];
+    pdl_wait();
     if (d.sync || d.ef == nullptr)
         return;
     const int64_t n = d.rows * d.cols;
@@ -1091,13 +1096,11 @@ int launch_gemm(dpo_muon_ctx *c, const GemmJob *jobs, int n_jobs, bool b_mn, cud
     // one CTA pair per co-resident cluster slot (the tile walk assumes every
     // pair runs at once)
     const int grid = 2 * (int)std::min<int64_t>(tiles, std::max(1, c->gemm_pairs));
-    if (b_mn)
-        dpo::gemm::ns_gemm_kernel<true><<<grid, dpo::gemm::kThreads, dpo::gemm::kSmemBytes, s>>>(L);
-    else
-        dpo::gemm::ns_gemm_kernel<false><<<grid, dpo::gemm::kThreads, dpo::gemm::kSmemBytes, s>>>(L);
+    const cudaError_t e =
+        dpo::launch_pdl(b_mn ? dpo::gemm::ns_gemm_kernel<true> : dpo::gemm::ns_gemm_kernel<false>,
+                        dim3(grid), dpo::gemm::kThreads, dpo::gemm::kSmemBytes, s, L);
     if (c->timing)
         ++c->gemm_launches;
-    const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? DPO_OK : mcuda(c, e, "Newton-Schulz GEMM launch");
 }
 
@@ -1123,18 +1126,18 @@ int orthogonalize(dpo_muon_ctx *c, cudaStream_t s, bool predict)
     ma.eps = c->hp.ns_eps;
     ma.inv_norm = c->d_inv_norm;
     ma.predict = predict ? 1 : 0;
-    const unsigned mgrid = (unsigned)c->n_chunks;
-    if (c->grad_dt == DPO_BF16)
-        dpo::muon::muon_momentum_kernel<__nv_bfloat16><<<mgrid, kThreads, 0, s>>>(ma);
-    else
-        dpo::muon::muon_momentum_kernel<float><<<mgrid, kThreads, 0, s>>>(ma);
-    cudaError_t e = cudaGetLastError();
+    const dim3 mgrid((unsigned)c->n_chunks);
+    cudaError_t e = dpo::launch_pdl(c->grad_dt == DPO_BF16
+                                        ? dpo::muon::muon_momentum_kernel<__nv_bfloat16>
+                                        : dpo::muon::muon_momentum_kernel<float>,
+                                    mgrid, kThreads, 0, s, ma);
     if (e != cudaSuccess)
         return mcuda(c, e, "momentum launch");
     const dpo::muon::NormalizeArgs na{c->d_mats, c->d_tile_begin, c->n, c->d_inv_norm,
                                       c->hp.ns_steps == 0 ? 1 : 0, predict ? 1 : 0};
-    dpo::muon::muon_normalize_kernel<<<(unsigned)c->n_tiles, kThreads, 0, s>>>(na);
-    if ((e = cudaGetLastError()) != cudaSuccess)
+    e = dpo::launch_pdl(dpo::muon::muon_normalize_kernel, dim3((unsigned)c->n_tiles), kThreads, 0,
+                        s, na);
+    if (e != cudaSuccess)
         return mcuda(c, e, "normalize launch");
     cudaEvent_t ev_end = nullptr;
     if (c->timing && c->hp.ns_steps > 0) {
@@ -1231,9 +1234,8 @@ extern "C" int dpo_muon_step(dpo_muon_ctx *c, float lr, void *stream)
     const int64_t k = c->k + 1;
     if (c->n == 0 || c->total_elems == 0) {
         if (c->capturable) {   // keep the device counter in step
-            dpo::muon::muon_scalars_kernel<<<1, 1, 0, s>>>(c->d_cnt, c->lr_src, lr, 0.0, 0,
-                                                           c->d_asc);
-            const cudaError_t e = cudaGetLastError();
+            const cudaError_t e = dpo::launch_pdl(dpo::muon::muon_scalars_kernel, dim3(1), 1, 0, s,
+                                                  c->d_cnt, c->lr_src, lr, 0.0, 0, c->d_asc);
             return e == cudaSuccess ? DPO_OK : mcuda(c, e, "scalars launch");
         }
         c->k = k;
@@ -1262,7 +1264,7 @@ extern "C" int dpo_muon_step(dpo_muon_ctx *c, float lr, void *stream)
     if (rc != DPO_OK)
         return rc;
     cudaError_t e;
-    const unsigned mgrid = (unsigned)c->n_chunks;
+    const dim3 mgrid((unsigned)c->n_chunks);
 
     // update, stash, history, weights
     const int64_t t = k - c->phase_k0;   // Alg. 1 iteration within the delayed phase
@@ -1279,29 +1281,27 @@ extern "C" int dpo_muon_step(dpo_muon_ctx *c, float lr, void *stream)
     aa.ef_now = aa.hist && !aa.sapipe && t >= 2 && c->hp.ef_lambda != 0.0f;
     aa.lam = c->hp.ef_lambda;
     if (c->capturable) {   // lr and EF's start from the device counters
-        dpo::muon::muon_scalars_kernel<<<1, 1, 0, s>>>(
-            c->d_cnt, c->lr_src, lr, (double)c->hp.weight_decay,
-            aa.hist && !aa.sapipe && c->hp.ef_lambda != 0.0f ? 1 : 0, c->d_asc);
-        if ((e = cudaGetLastError()) != cudaSuccess)
+        e = dpo::launch_pdl(dpo::muon::muon_scalars_kernel, dim3(1), 1, 0, s, c->d_cnt, c->lr_src,
+                            lr, (double)c->hp.weight_decay,
+                            aa.hist && !aa.sapipe && c->hp.ef_lambda != 0.0f ? 1 : 0, c->d_asc);
+        if (e != cudaSuccess)
             return mcuda(c, e, "scalars launch");
         aa.dev = c->d_asc;
     }
     const bool st = c->hp.delay == 1;
-    if (!st)
-        dpo::muon::muon_apply_kernel<dpo::kStashNone><<<mgrid, kThreads, 0, s>>>(aa);
-    else if (c->stash_dt == DPO_BF16)
-        dpo::muon::muon_apply_kernel<dpo::kStashBF16><<<mgrid, kThreads, 0, s>>>(aa);
-    else
-        dpo::muon::muon_apply_kernel<dpo::kStashF32><<<mgrid, kThreads, 0, s>>>(aa);
-    if ((e = cudaGetLastError()) != cudaSuccess)
+    e = dpo::launch_pdl(!st ? dpo::muon::muon_apply_kernel<dpo::kStashNone>
+                        : c->stash_dt == DPO_BF16 ? dpo::muon::muon_apply_kernel<dpo::kStashBF16>
+                                                  : dpo::muon::muon_apply_kernel<dpo::kStashF32>,
+                        mgrid, kThreads, 0, s, aa);
+    if (e != cudaSuccess)
         return mcuda(c, e, "apply launch");
     if (updated && aa.hist) {
         // SAPipe-WP updated state: the step once more on the same gradient
         // from the momentum just stored, decaying X_{t+1}, into the history
         if ((rc = orthogonalize(c, s, true)) != DPO_OK)
             return rc;
-        dpo::muon::muon_predict_kernel<<<mgrid, kThreads, 0, s>>>(aa);
-        if ((e = cudaGetLastError()) != cudaSuccess)
+        if ((e = dpo::launch_pdl(dpo::muon::muon_predict_kernel, mgrid, kThreads, 0, s, aa)) !=
+            cudaSuccess)
             return mcuda(c, e, "prediction launch");
     }
     if (!c->capturable)

@@ -145,6 +145,13 @@ __global__ void __launch_bounds__(kStepThreads) fused_step_kernel(const StepArgs
 
     const int64_t stride = (int64_t)gridDim.x * kStepThreads;
     int64_t p = (int64_t)blockIdx.x * kStepThreads + threadIdx.x;
+    Cursor c;
+    DevTensor d{};
+    if (p < a.total_pkts) {   // the tables are constant: found before the wait
+        c.seek(a.pkt_begin, a.n_tensors, p);
+        d = a.table[c.t];
+    }
+    pdl_wait();
     if (p >= a.total_pkts)
         return;
 
@@ -165,9 +172,6 @@ __global__ void __launch_bounds__(kStepThreads) fused_step_kernel(const StepArgs
     const bool ef_now = CORR == kCorrEF && sc.lam != 0.0f;
     const float dc = a.dc_lambda;
 
-    Cursor c;
-    c.seek(a.pkt_begin, a.n_tensors, p);
-    DevTensor d = a.table[c.t];
     for (; p < a.total_pkts; p += stride) {
         if (c.advance(a.pkt_begin, p))
             d = a.table[c.t];
