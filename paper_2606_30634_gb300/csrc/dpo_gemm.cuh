@@ -257,80 +257,76 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
     return *reinterpret_cast<const uint32_t *>(&h);
 }
 
-// Tile t of a launch: batch entry, row block and column block. A full
-// product walks bands of kBandRows block rows (all of them, up to 4096 rows),
-// each band column by column, so the tiles in flight at once (one per CTA
-// pair) share the band's A row blocks and a few B column blocks in L2, and
-// each B column block comes from DRAM about once per band. On a 4096 x 11008
-// operand, walking whole block rows instead had the pairs stream all 43 B
-// column blocks every round. A symmetric product (sym, m_tiles == n_tiles)
-// enumerates only the tiles on or above the diagonal, column by column
-// (column n holds n + 1 of them), so the pairs' shares of its work differ by
-// at most one tile, and the tiles in flight at once read the first block rows
-// of the operand before the pairs move on to the last ones.
+// The order in which a launch's tiles of one product go out. A full product
+// walks bands of kBandRows block rows (all of them, up to 4096 rows), each
+// band column by column, so the tiles in flight at once (one per CTA pair)
+// share the band's A row blocks and a few B column blocks in L2, and each B
+// column block comes from DRAM about once per band. On a 4096 x 11008 operand,
+// walking whole block rows instead had the pairs stream all 43 B column blocks
+// every round. A symmetric product (sym, m_tiles == n_tiles) enumerates only
+// the tiles on or above the diagonal, column by column (column n holds n + 1
+// of them), so the pairs' shares of its work differ by at most one tile, and
+// the tiles in flight at once read the first block rows of the operand before
+// the pairs move on to the last ones.
 constexpr int kBandRows = 16;   // block rows per band of a full product's walk
 
 struct TileGrid {
     int m_tiles, n_tiles, nb, sym;
-    __host__ __device__ __forceinline__ int per_batch() const
+    int per_batch() const { return sym ? m_tiles * (m_tiles + 1) / 2 : m_tiles * n_tiles; }
+    int count() const { return per_batch() * nb; }
+    // fn(batch entry, first row, first column) for every tile in order
+    template <class F>
+    void walk(F &&fn) const
     {
-        return sym ? m_tiles * (m_tiles + 1) / 2 : m_tiles * n_tiles;
-    }
-    __host__ __device__ __forceinline__ int count() const { return per_batch() * nb; }
-    __device__ __forceinline__ void at(int t, int &b, int &m0, int &n0) const
-    {
-        const int per = per_batch();
-        b = t / per;
-        int u = t - b * per;
-        if (sym) {
-            int n = 0;
-            while (u > n) {   // u < per, so n stays below m_tiles
-                u -= n + 1;
-                ++n;
+        for (int b = 0; b < nb; ++b) {
+            if (sym) {
+                for (int n = 0; n < n_tiles; ++n)
+                    for (int m = 0; m <= n; ++m)
+                        fn(b, m * TM, n * TN);
+            } else {
+                for (int first = 0; first < m_tiles; first += kBandRows)
+                    for (int n = 0; n < n_tiles; ++n)
+                        for (int m = first; m < m_tiles && m < first + kBandRows; ++m)
+                            fn(b, m * TM, n * TN);
             }
-            m0 = u * TM;
-            n0 = n * TN;
-        } else {
-            const int band = u / (kBandRows * n_tiles);
-            const int first = band * kBandRows;
-            const int rows = min(kBandRows, m_tiles - first);
-            const int r = u - first * n_tiles;   // 0 <= r < rows * n_tiles
-            m0 = (first + r % rows) * TM;
-            n0 = (r / rows) * TN;
         }
     }
 };
 
 // One launch computes the same product for up to kMaxGroups batches of
 // different shapes (the shape groups of a Newton-Schulz step): each group
-// has its own operand and output maps, epilogue and tile grid, and its tiles
-// follow the previous group's in the launch's order. Small sets then fill
-// the CTA pairs with one launch per product instead of one per shape.
+// has its own operand and output maps and epilogue, and its tiles follow the
+// previous group's in the launch's order. Small sets then fill the CTA pairs
+// with one launch per product instead of one per shape.
 constexpr int kMaxGroups = 4;
 
 struct GemmGroup {
     CUtensorMap a, b, d, dt;   // A, B (operands), D and D^T (stores)
     Params p;
-    TileGrid tg;
-    int tile0;                 // first tile of this group in the launch
 };
 
+// The tiles come from a table made at init: x the group, y the batch entry,
+// z and w the tile's first row and column. Each role of the kernel reads its
+// pair's next entry while it works on the current one. Deriving them from t
+// in the kernel (a search over the groups, four divisions) read the launch's
+// parameters through dependent loads and took every role, the MMA lane among
+// them, some 3,900 cycles per tile: a third of a K = 768 tile's time.
 struct GemmLaunch {
     GemmGroup g[kMaxGroups];
+    const int4 *tiles;
     int n_groups;
     int n_tiles;               // over all groups
 };
 
-// Group, batch entry, row block and column block of tile t of a launch.
-__device__ __forceinline__ const GemmGroup &locate(const GemmLaunch &L, int t, int &b, int &m0,
-                                                   int &n0)
+// Entry t of the tile table, pinned where it is written (a plain load may be
+// moved down to its first use, a tile later).
+__device__ __forceinline__ int4 load_tile(const int4 *p)
 {
-    int gi = L.n_groups - 1;
-    while (gi > 0 && t < L.g[gi].tile0)
-        --gi;
-    const GemmGroup &G = L.g[gi];
-    G.tg.at(t - G.tile0, b, m0, n0);
-    return G;
+    int4 q;
+    asm volatile("ld.global.nc.v4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(q.x), "=r"(q.y), "=r"(q.z), "=r"(q.w)
+                 : "l"(p));
+    return q;
 }
 
 // Persistent: the CTA pairs (clusters of 2) take tiles c, c + pairs, ...
@@ -348,11 +344,13 @@ template <bool BMN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     ns_gemm_kernel(const __grid_constant__ GemmLaunch L)
 {
-    const Params &p0 = L.g[0].p;   // err and stall are the launch's
+    unsigned int *const err = L.g[0].p.err;   // err and stall are the launch's
+    const int stall = L.g[0].p.stall;
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bars[2 * kStages + 4];
     __shared__ uint32_t tmem_slot;
     __shared__ int aborted;
+    __shared__ Params params[kMaxGroups];   // read per tile, by every role
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
@@ -377,6 +375,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             mbar_init(acc_empty(a), 8);   // one arrival per epilogue warp of the pair
         }
         aborted = 0;
+#pragma unroll
+        for (int gi = 0; gi < kMaxGroups; ++gi)
+            params[gi] = L.g[gi].p;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {   // both CTAs of the pair allocate together
@@ -391,6 +392,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
     const int n_tiles = L.n_tiles;
+    const int4 *const tiles = L.tiles;
+    int4 next = {0, 0, 0, 0};   // this pair's next tile (constant table: read before the wait)
+    if (pair < n_tiles)
+        next = load_tile(tiles + pair);
     pdl_wait();
 
     if (warp == 0) {
@@ -403,16 +408,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             }
             int it = 0;   // k-blocks issued by this CTA
             for (int t = pair; t < n_tiles && !*(volatile int *)&aborted; t += n_pairs) {
-                int b, m0, n0;
-                const GemmGroup &G = locate(L, t, b, m0, n0);
-                const CUtensorMap *tma_a = &G.a, *tma_b = &G.b;
-                const int kb_n = G.p.k_blocks;
+                const int gi = next.x, b = next.y, m0 = next.z, n0 = next.w;
+                if (t + n_pairs < n_tiles)
+                    next = load_tile(tiles + t + n_pairs);
+                const CUtensorMap *tma_a = &L.g[gi].a, *tma_b = &L.g[gi].b;
+                const int kb_n = params[gi].k_blocks;
                 const int ma = m0 + (int)rank * BM, nb_ = n0 + (int)rank * BH;
                 for (int kb = 0; kb < kb_n; ++kb, ++it) {
                     const int s = it % kStages;
                     const uint32_t ph = (uint32_t)(it / kStages) & 1u;
                     if (!mbar_wait(empty(s), ph ^ 1u) || *(volatile int *)&aborted) {
-                        atomicOr(p0.err, kErrWaitEmpty);
+                        atomicOr(err, kErrWaitEmpty);
                         aborted = 1;
                         break;
                     }
@@ -440,18 +446,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             if (leader)
                 for (int q = it - kStages < 0 ? 0 : it - kStages; q < it; ++q)
                     if (!mbar_wait(full(q % kStages), (uint32_t)(q / kStages) & 1u))
-                        atomicOr(p0.err, kErrDrain);
+                        atomicOr(err, kErrDrain);
         }
     } else if (warp == 1) {
         if (lane == 0 && leader) {
             int it = 0, lt = 0;   // k-blocks consumed, tiles accumulated
             for (int t = pair; t < n_tiles && !*(volatile int *)&aborted; t += n_pairs) {
-                int b, m0, n0;
-                const int kb_n = locate(L, t, b, m0, n0).p.k_blocks;
+                const int kb_n = params[next.x].k_blocks;
+                if (t + n_pairs < n_tiles)
+                    next = load_tile(tiles + t + n_pairs);
                 const int a = lt & 1;
                 const uint32_t aph = (uint32_t)(lt >> 1) & 1u;
-                if (!mbar_wait(acc_empty(a), p0.stall && lt == 0 ? aph : aph ^ 1u)) {
-                    atomicOr(p0.err, kErrWaitDone);
+                if (!mbar_wait(acc_empty(a), stall && lt == 0 ? aph : aph ^ 1u)) {
+                    atomicOr(err, kErrWaitDone);
                     aborted = 1;
                     break;
                 }
@@ -462,7 +469,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                     const int s = it % kStages;
                     const uint32_t ph = (uint32_t)(it / kStages) & 1u;
                     if (!mbar_wait(full(s), ph) || *(volatile int *)&aborted) {
-                        atomicOr(p0.err, kErrWaitFull);
+                        atomicOr(err, kErrWaitFull);
                         aborted = 1;
                         ok = false;
                         break;
@@ -486,7 +493,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                     // the MMAs issued for this tile finish before the pair
                     // leaves and its TMEM is released
                     if (!mbar_wait(acc_full(a), aph))
-                        atomicOr(p0.err, kErrDrain);
+                        atomicOr(err, kErrDrain);
                     break;
                 }
             }
@@ -514,9 +521,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const int crs = lane >> 2, cg = lane & 3;   // coalesced load: sub-row, granule
         int lt = 0, staged = 0;
         for (int t = pair; t < n_tiles; t += n_pairs) {
-            int b, m0, n0;
-            const GemmGroup &G = locate(L, t, b, m0, n0);
-            const Params &p = G.p;
+            const int gi = next.x, b = next.y, m0 = next.z, n0 = next.w;
+            if (t + n_pairs < n_tiles)
+                next = load_tile(tiles + t + n_pairs);
+            const GemmGroup &G = L.g[gi];
+            const Params p = params[gi];   // in registers: the asm statements below clobber memory
             const int a = lt & 1;
             const int row0 = m0 + (int)rank * BM + q * 32;
             // C at (row0 + crs, n0 + 8 cg); rows 8 i further for i = 0..3
@@ -535,7 +544,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             }
             const bool seen = mbar_wait(acc_full(a), (uint32_t)(lt >> 1) & 1u);
             if (!seen)
-                atomicOr(p0.err, kErrWaitDone);
+                atomicOr(err, kErrWaitDone);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             // tcgen05.ld is warp-collective: the whole warp goes on, or none of it.
             if (!__all_sync(0xFFFFFFFFu, seen && !*(volatile int *)&aborted))

@@ -569,6 +569,19 @@ bool make_store_map(CUtensorMap *m, void *base, int64_t rows, int64_t cols, int6
 
 int64_t pad_up(int64_t v) { return (v + kPad - 1) / kPad * kPad; }
 
+// One Newton-Schulz launch set: up to kMaxGroups shape groups that share each
+// product's launch, and per product (X X^T, c A A + b A, B X + a X) the order
+// of its groups and its part of the tile table.
+struct LaunchSet {
+    int n = 0;
+    int group[dpo::gemm::kMaxGroups];
+    struct {
+        int order[dpo::gemm::kMaxGroups];   // positions in group[]
+        int64_t first = 0;                  // first entry of the tile table
+        int tiles = 0;
+    } prod[3];
+};
+
 struct Group {
     int64_t r, w, R, W;
     std::vector<int> mats;
@@ -605,6 +618,8 @@ struct dpo_muon_ctx {
     std::vector<dpo_matrix> mats;
     std::vector<DevMat> host_mats;
     std::vector<Group> groups;
+    std::vector<LaunchSet> sets;
+    int4 *d_tiles = nullptr;          // tile table of every set and product
     int n_chunks = 0;         // CTAs of the momentum, update and prediction passes
     int chunk_elems = 0;
     int n_tiles = 0;          // CTAs of the normalisation
@@ -820,6 +835,71 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
             g.has_tall = g.has_tall || mats[mi].rows > mats[mi].cols;
     }
     c->ws_bytes = ws;
+    // CTA pairs the GEMM kernels keep resident at once (a failure is reported
+    // after the allocations, where the launches it stops would come).
+    c->gemm_pairs = 1 << 30;
+    cudaError_t e_gemm = cudaSuccess;
+    for (const void *fn : {(const void *)dpo::gemm::ns_gemm_kernel<false>,
+                           (const void *)dpo::gemm::ns_gemm_kernel<true>}) {
+        e_gemm = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      dpo::gemm::kSmemBytes);
+        int pairs = 0;
+        if (e_gemm == cudaSuccess) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(2 * std::max(1, c->sms / 2));
+            cfg.blockDim = dim3(dpo::gemm::kThreads);
+            cfg.dynamicSmemBytes = dpo::gemm::kSmemBytes;
+            e_gemm = cudaOccupancyMaxActiveClusters(&pairs, fn, &cfg);
+        }
+        if (e_gemm != cudaSuccess)
+            break;
+        c->gemm_pairs = std::min(c->gemm_pairs, pairs);
+    }
+    // When some shape group's launches are short (at most 16 rounds of tiles
+    // over the CTA pairs), each product of a Newton-Schulz step covers all
+    // shape groups in one launch: one group's tiles fill the pairs another
+    // leaves idle, and a step takes 3 launches instead of 3 per group (GPT-2:
+    // every group short; the Llama-1B set's 512 x 2048 group: 20.08 -> 19.80
+    // ms of GEMMs per step on GB300). Sets whose groups are all long keep one
+    // group per launch and run the groups' chains one after another (7B set:
+    // 0.3% slower grouped; two chains at once on two streams mixed their
+    // operands in L2, 336 -> 410 ms per step).
+    int64_t min_tiles = INT64_MAX;
+    for (const Group &g : c->groups)
+        min_tiles = std::min<int64_t>(min_tiles, (int64_t)g.mats.size() *
+                                                     (g.R / dpo::gemm::TM) * (g.W / dpo::gemm::TN));
+    c->grouped = c->groups.size() > 1 && min_tiles <= 16 * (int64_t)std::max(1, c->gemm_pairs);
+    // Launch sets and their tile tables. A launch takes its groups with more K
+    // blocks first: the pairs take tiles round-robin, so the longest tiles go
+    // out first and the short ones fill the last round.
+    std::vector<int4> tiles;
+    const int per_set = c->grouped ? dpo::gemm::kMaxGroups : 1;
+    for (int g0 = 0; g0 < (int)c->groups.size(); g0 += per_set) {
+        LaunchSet ls;
+        ls.n = std::min(per_set, (int)c->groups.size() - g0);
+        for (int q = 0; q < ls.n; ++q)
+            ls.group[q] = g0 + q;
+        for (int prod = 0; prod < 3; ++prod) {
+            auto &p = ls.prod[prod];
+            auto k_of = [&](int q) {
+                const Group &g = c->groups[ls.group[q]];
+                return prod == 0 ? g.W : g.R;
+            };
+            for (int q = 0; q < ls.n; ++q)
+                p.order[q] = q;
+            std::stable_sort(p.order, p.order + ls.n, [&](int x, int y) { return k_of(x) > k_of(y); });
+            p.first = (int64_t)tiles.size();
+            for (int q = 0; q < ls.n; ++q) {
+                const Group &g = c->groups[ls.group[p.order[q]]];
+                const dpo::gemm::TileGrid tg{(int)(g.R / dpo::gemm::TM),
+                                             (int)((prod == 2 ? g.W : g.R) / dpo::gemm::TN),
+                                             (int)g.mats.size(), prod != 2};
+                tg.walk([&](int b, int m0, int n0) { tiles.push_back(make_int4(q, b, m0, n0)); });
+            }
+            p.tiles = (int)((int64_t)tiles.size() - p.first);
+        }
+        c->sets.push_back(ls);
+    }
     // Norm-pass table (the elementwise path's gradient-norm kernel).
     int64_t total_pkts = 0;
     std::vector<int64_t> pkt_begin(n + 1, 0);
@@ -839,7 +919,7 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
 
     // Device block: mats | partials | chunk and tile prefixes | tickets |
     // inv_norm | err | norm table | pkt_begin | norm partials | norm scalars |
-    // capturable counters and scalars.
+    // capturable counters and scalars | GEMM tile table.
     auto al = [](int64_t v) { return (v + 255) / 256 * 256; };
     int64_t off = 0;
     const int64_t o_mats = off;
@@ -868,6 +948,8 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
     off += al(sizeof(dpo::muon::MuonCounters));
     const int64_t o_asc = off;
     off += al(sizeof(dpo::muon::ApplyScalars));
+    const int64_t o_tiles = off;
+    off += al((int64_t)(sizeof(int4) * std::max<size_t>(1, tiles.size())));
 
     cudaError_t e = dpo::device_alloc(&c->dev_block, (size_t)off);
     if (e != cudaSuccess) {
@@ -896,6 +978,7 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
     c->d_norm_scalars = reinterpret_cast<dpo::NormScalars *>(blk + o_nsc);
     c->d_cnt = reinterpret_cast<dpo::muon::MuonCounters *>(blk + o_cnt);
     c->d_asc = reinterpret_cast<dpo::muon::ApplyScalars *>(blk + o_asc);
+    c->d_tiles = reinterpret_cast<int4 *>(blk + o_tiles);
 
     // Carve the workspace and build the tensor maps.
     char *wp = static_cast<char *>(c->ws);
@@ -988,6 +1071,7 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
     MUON_COPY(c->d_norm_table, ntab.data(), sizeof(dpo::DevTensor) * n);
     MUON_COPY(c->d_pkt_begin, pkt_begin.data(), sizeof(int64_t) * (n + 1));
     MUON_COPY(c->d_chunk_begin, chunk_begin.data(), sizeof(int) * (n + 1));
+    MUON_COPY(c->d_tiles, tiles.data(), sizeof(int4) * tiles.size());
     MUON_COPY(c->d_tile_begin, tile_begin.data(), sizeof(int) * (n + 1));
 #undef MUON_COPY
     e = cudaMemsetAsync(c->d_err, 0, sizeof(unsigned int), s);
@@ -1001,42 +1085,11 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
         free_ctx(c);
         return mcuda(nullptr, e, "workspace clear");
     }
-    c->gemm_pairs = 1 << 30;
-    for (const void *fn : {(const void *)dpo::gemm::ns_gemm_kernel<false>,
-                           (const void *)dpo::gemm::ns_gemm_kernel<true>}) {
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 dpo::gemm::kSmemBytes);
-        int pairs = 0;
-        if (e == cudaSuccess) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(2 * std::max(1, c->sms / 2));
-            cfg.blockDim = dim3(dpo::gemm::kThreads);
-            cfg.dynamicSmemBytes = dpo::gemm::kSmemBytes;
-            e = cudaOccupancyMaxActiveClusters(&pairs, fn, &cfg);
-        }
-        if (e != cudaSuccess)
-            break;
-        c->gemm_pairs = std::min(c->gemm_pairs, pairs);
-    }
-    if (e != cudaSuccess || c->gemm_pairs < 1) {
+    if (e_gemm != cudaSuccess || c->gemm_pairs < 1) {
         free_ctx(c);
-        return e != cudaSuccess ? mcuda(nullptr, e, "GEMM launch configuration")
-                                : mfail(nullptr, DPO_ECUDA, "GEMM kernel cannot be resident");
+        return e_gemm != cudaSuccess ? mcuda(nullptr, e_gemm, "GEMM launch configuration")
+                                     : mfail(nullptr, DPO_ECUDA, "GEMM kernel cannot be resident");
     }
-    // When some shape group's launches are short (at most 16 rounds of tiles
-    // over the CTA pairs), each product of a Newton-Schulz step covers all
-    // shape groups in one launch: one group's tiles fill the pairs another
-    // leaves idle, and a step takes 3 launches instead of 3 per group (GPT-2:
-    // every group short; the Llama-1B set's 512 x 2048 group: 20.08 -> 19.80
-    // ms of GEMMs per step on GB300). Sets whose groups are all long keep one
-    // group per launch and run the groups' chains one after another (7B set:
-    // 0.3% slower grouped; two chains at once on two streams mixed their
-    // operands in L2, 336 -> 410 ms per step).
-    int64_t min_tiles = INT64_MAX;
-    for (const Group &g : c->groups)
-        min_tiles = std::min<int64_t>(min_tiles, (int64_t)g.mats.size() *
-                                                     (g.R / dpo::gemm::TM) * (g.W / dpo::gemm::TN));
-    c->grouped = c->groups.size() > 1 && min_tiles <= 16 * (int64_t)std::max(1, c->gemm_pairs);
     if (init_mode == DPO_INIT_FRESH) {
         const int rc = launch_init(c, s, 1, 1);
         if (rc != DPO_OK) {
@@ -1055,47 +1108,31 @@ namespace {
 struct GemmJob {
     const CUtensorMap *ta, *tb, *td, *tdt;
     dpo::gemm::Params p;
-    int64_t M, N, nb;
 };
 
-// One launch over up to kMaxGroups jobs of the same product (all read B
-// K-major, or all MN-major), the jobs with more K blocks first: the pairs
-// take tiles round-robin, so the longest tiles go out first and the short
-// ones fill the last round.
-int launch_gemm(dpo_muon_ctx *c, const GemmJob *jobs, int n_jobs, bool b_mn, cudaStream_t s)
+// One launch over the jobs of one product of a launch set (all read B K-major,
+// or all MN-major), in the order of its tile table.
+int launch_gemm(dpo_muon_ctx *c, const LaunchSet &ls, int prod, const GemmJob *jobs, cudaStream_t s)
 {
-    if (n_jobs < 1 || n_jobs > dpo::gemm::kMaxGroups)
-        return mfail(c, DPO_EINVAL, "GEMM launch of %d groups", n_jobs);
-    int order[dpo::gemm::kMaxGroups];
-    for (int j = 0; j < n_jobs; ++j)
-        order[j] = j;
-    std::stable_sort(order, order + n_jobs, [&](int x, int y) {
-        return jobs[x].p.k_blocks > jobs[y].p.k_blocks;
-    });
+    const auto &pr = ls.prod[prod];
     dpo::gemm::GemmLaunch L;
     std::memset(&L, 0, sizeof L);
-    int64_t tiles = 0;
-    for (int q = 0; q < n_jobs; ++q) {
-        const GemmJob &j = jobs[order[q]];
-        dpo::gemm::TileGrid tg{(int)(j.M / dpo::gemm::TM), (int)(j.N / dpo::gemm::TN), (int)j.nb,
-                               j.p.sym};
-        if (j.p.sym && j.M != j.N)
-            return mfail(c, DPO_EINVAL, "symmetric product of a non-square shape");
+    for (int q = 0; q < ls.n; ++q) {
+        const GemmJob &j = jobs[pr.order[q]];
         dpo::gemm::GemmGroup &G = L.g[q];
         G.a = *j.ta;
         G.b = *j.tb;
         G.d = *j.td;
         G.dt = *j.tdt;
         G.p = j.p;
-        G.tg = tg;
-        G.tile0 = (int)tiles;
-        tiles += tg.count();
     }
-    L.n_groups = n_jobs;
-    L.n_tiles = (int)tiles;
+    L.tiles = c->d_tiles + pr.first;
+    L.n_groups = ls.n;
+    L.n_tiles = pr.tiles;
+    const bool b_mn = prod == 2;
     // one CTA pair per co-resident cluster slot (the tile walk assumes every
     // pair runs at once)
-    const int grid = 2 * (int)std::min<int64_t>(tiles, std::max(1, c->gemm_pairs));
+    const int grid = 2 * std::min(pr.tiles, std::max(1, c->gemm_pairs));
     const cudaError_t e =
         dpo::launch_pdl(b_mn ? dpo::gemm::ns_gemm_kernel<true> : dpo::gemm::ns_gemm_kernel<false>,
                         dim3(grid), dpo::gemm::kThreads, dpo::gemm::kSmemBytes, s, L);
@@ -1164,19 +1201,15 @@ int orthogonalize(dpo_muon_ctx *c, cudaStream_t s, bool predict)
         --c->stall_launches;
         return 1;
     };
-    const int n_groups = (int)c->groups.size();
-    const int per = c->grouped ? dpo::gemm::kMaxGroups : 1;
-    for (int g0 = 0; g0 < n_groups; g0 += per) {
-        const int n = std::min(per, n_groups - g0);
+    for (const LaunchSet &ls : c->sets) {
         for (int it = 0; it < c->hp.ns_steps; ++it) {
             const bool last = it + 1 == c->hp.ns_steps;
             const int cur = it % 2, nxt = cur ^ 1;
             GemmJob xx[dpo::gemm::kMaxGroups], aa[dpo::gemm::kMaxGroups],
                 bx[dpo::gemm::kMaxGroups];
             const int st_xx = stall_next(), st_aa = stall_next(), st_bx = stall_next();
-            for (int q = 0; q < n; ++q) {
-                Group &g = c->groups[g0 + q];
-                const int64_t nb = (int64_t)g.mats.size();
+            for (int q = 0; q < ls.n; ++q) {
+                Group &g = c->groups[ls.group[q]];
                 dpo::gemm::Params p{};
                 p.err = c->d_err;
                 // A = X X^T
@@ -1184,7 +1217,7 @@ int orthogonalize(dpo_muon_ctx *c, cudaStream_t s, bool predict)
                 p.k_blocks = (int)(g.W / dpo::gemm::BK);
                 p.sym = 1;
                 p.stall = st_xx;
-                xx[q] = GemmJob{&g.x128[cur], &g.x128[cur], &g.st_a, &g.st_a, p, g.R, g.R, nb};
+                xx[q] = GemmJob{&g.x128[cur], &g.x128[cur], &g.st_a, &g.st_a, p};
                 // B = c A A + b A
                 p.c = g.a;
                 p.ldc = g.R;
@@ -1193,7 +1226,7 @@ int orthogonalize(dpo_muon_ctx *c, cudaStream_t s, bool predict)
                 p.beta = c->hp.ns_b;
                 p.k_blocks = (int)(g.R / dpo::gemm::BK);
                 p.stall = st_aa;
-                aa[q] = GemmJob{&g.a128, &g.a128, &g.st_b, &g.st_b, p, g.R, g.R, nb};
+                aa[q] = GemmJob{&g.a128, &g.a128, &g.st_b, &g.st_b, p};
                 // X <- B X + a X (X read MN-major in place of X^T), and at the
                 // last step X^T for the tall matrices' output
                 p.sym = 0;
@@ -1205,13 +1238,13 @@ int orthogonalize(dpo_muon_ctx *c, cudaStream_t s, bool predict)
                 p.beta = c->hp.ns_a;
                 p.k_blocks = (int)(g.R / dpo::gemm::BK);
                 p.stall = st_bx;
-                bx[q] = GemmJob{&g.b128, &g.x_mn[cur], &g.st_x[nxt], &g.st_xt, p, g.R, g.W, nb};
+                bx[q] = GemmJob{&g.b128, &g.x_mn[cur], &g.st_x[nxt], &g.st_xt, p};
             }
-            int rc = launch_gemm(c, xx, n, false, s);
+            int rc = launch_gemm(c, ls, 0, xx, s);
             if (rc == DPO_OK)
-                rc = launch_gemm(c, aa, n, false, s);
+                rc = launch_gemm(c, ls, 1, aa, s);
             if (rc == DPO_OK)
-                rc = launch_gemm(c, bx, n, true, s);
+                rc = launch_gemm(c, ls, 2, bx, s);
             if (rc != DPO_OK)
                 return rc;
         }
