@@ -19,7 +19,7 @@
 //               tcgen05.mma.cta_group::2.kind::f16 (M 256, N 256, K 16) eight
 //               times per stage, reading both CTAs' halves, and commits each
 //               stage and each finished tile to both CTAs;
-//   warps 2-5   epilogue of this CTA's 128 rows: tcgen05.ld 32 lanes x 32
+//   warps 2-9   epilogue of this CTA's 128 rows: tcgen05.ld 32 lanes x 32
 //               columns at a time, scale, add the addend, round to bf16,
 //               stage the 32 x 32 chunk (and, when asked, its transpose) in
 //               shared memory and write it with a TMA store.
@@ -52,16 +52,24 @@ namespace gemm {
 // span); eight MMAs per stage halve the barrier hand-offs per MMA against
 // 64-wide stages, which measured 10% faster on GB300 at equal ring size.
 constexpr int TM = 256, TN = 256, BM = 128, BH = 128, BK = 128, kBoxK = 64, kStages = 3;
-constexpr int kThreads = 192;
+// Epilogue warps: two per TMEM lane quarter, each taking half of the tile's
+// columns: a tile's epilogue is a serial chain per warp (TMEM read, addend,
+// staging, store), which the 6 k-blocks of a K = 768 tile do not hide at four
+// warps. GB300, four against eight warps, whole step: GPT-2 1816 -> 1777 us,
+// twelve 768-wide layers 1525 -> 1486, two 256x768 matrices 145 -> 133; a 7B
+// layer, whose tiles have 32 k-blocks, is unchanged.
+constexpr int kEpiWarps = 8;
+constexpr int kThreads = 64 + 32 * kEpiWarps;
+constexpr int kEpiCols = TN * 4 / kEpiWarps;   // columns per epilogue warp
 constexpr uint32_t kTmemCols = 256;                  // one accumulator (fp32, TN columns)
 constexpr int kABytes = BM * BK * 2;                 // 32 KiB
 constexpr int kBBytes = BH * BK * 2;                 // 32 KiB
 constexpr int kStageBytes = kABytes + kBBytes;       // 64 KiB per CTA
-// Epilogue staging behind the ring: per epilogue warp two buffers for its
-// 32 x 32 chunk of D and two for the chunk's transpose, 2 KiB each, in the
-// 64-byte-swizzled layout the TMA store reads.
+// Epilogue staging behind the ring: per epilogue warp two buffers of 2 KiB, in
+// the 64-byte-swizzled layout the TMA store reads: two 32 x 32 chunks of D in
+// turn, or one chunk of D and its transpose.
 constexpr int kChunkBytes = 32 * 32 * 2;
-constexpr int kEpiBytes = 4 * 4 * kChunkBytes;              // 32 KiB
+constexpr int kEpiBytes = kEpiWarps * 2 * kChunkBytes;      // 32 KiB
 // ring + 1024-byte alignment slack + staging
 constexpr int kSmemBytes = kStages * kStageBytes + 1024 + kEpiBytes;
 constexpr unsigned long long kWaitNs = 1000000000ull;  // 1 s per wait
@@ -318,6 +326,17 @@ struct GemmLaunch {
     int n_tiles;               // over all groups
 };
 
+// 16 bytes of the addend, pinned where it is written, before the wait for the
+// accumulator.
+__device__ __forceinline__ uint4 load_c(const __nv_bfloat16 *p)
+{
+    uint4 q;
+    asm volatile("ld.global.nc.v4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(q.x), "=r"(q.y), "=r"(q.z), "=r"(q.w)
+                 : "l"(p));
+    return q;
+}
+
 // Entry t of the tile table, pinned where it is written (a plain load may be
 // moved down to its first use, a tile later).
 __device__ __forceinline__ int4 load_tile(const int4 *p)
@@ -337,7 +356,7 @@ __device__ __forceinline__ int4 load_tile(const int4 *p)
 //   full[s]      (leader) both ranks' TMA bytes of stage s have landed
 //   empty[s]     (each)   the leader's MMAs have finished reading stage s
 //   acc_full[a]  (each)   accumulator a holds a finished tile
-//   acc_empty[a] (leader) all 8 epilogue warps of the pair have read it
+//   acc_empty[a] (leader) all epilogue warps of the pair have read it
 // BMN: the B operand is stored N-contiguous (a row-major K x N matrix) and
 // loaded as two 64 x 64 boxes per stage, read MN-major by the MMA.
 template <bool BMN>
@@ -372,7 +391,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(acc_full(a), 1);
-            mbar_init(acc_empty(a), 8);   // one arrival per epilogue warp of the pair
+            mbar_init(acc_empty(a), 2 * kEpiWarps);   // one arrival per epilogue warp of the pair
         }
         aborted = 0;
 #pragma unroll
@@ -500,47 +519,43 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         }
     } else {
         // Epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 = this CTA's
-        // tile rows m0 + BM rank + 32 (w % 4) + lane. Each 32 x 32 chunk is
-        // staged in shared memory (and its transpose, for a mirrored or a
-        // transposed output) and written by one TMA store per box from lane
-        // 0; direct stores from 32 rows at a time cost the MMAs a fifth of
-        // their rate on GB300. Two buffers per kind alternate, so lane 0
-        // waits for the group of two chunks back before they are rewritten.
-        const int q = warp & 3;
-        const uint32_t wbuf = ring + (uint32_t)(kStages * kStageBytes + q * 4 * kChunkBytes);
-        // The addend C (c A A + b A, B X + a X) is read kCPre chunks ahead of
-        // its use, the first ones before the accumulator is ready, coalesced:
-        // lane l loads granule l % 4 (8 columns) of rows l / 4 + 8 i of the
-        // warp's 32 x 32 chunk, 8 rows of 64 bytes per instruction; the chunk
-        // is then turned through its staging buffer so that each lane holds
-        // its own row. Loading each lane's own row instead touched 32 lines
-        // per instruction; where K is short (768) that made the chain 6 %
-        // slower on GB300, and where K is long the epilogue is hidden behind
-        // the MMAs either way. C is never the launch's output.
-        constexpr int kCPre = 4;
+        // tile rows m0 + BM rank + 32 (w % 4) + lane, and the half of the tile's
+        // columns that (w - 2) / 4 names. Each 32 x 32 chunk is staged in
+        // shared memory (and its transpose, for a mirrored or a transposed
+        // output) and written by one TMA store per box from lane 0; direct
+        // stores from 32 rows at a time cost the MMAs a fifth of their rate
+        // on GB300. Lane 0 waits until the buffers it is about to rewrite have
+        // been read.
+        const int q = warp & 3, half = (warp - 2) >> 2;
+        const uint32_t wbuf =
+            ring + (uint32_t)(kStages * kStageBytes + (warp - 2) * 2 * kChunkBytes);
+        // The addend C (c A A + b A, B X + a X) of all the warp's chunks is
+        // read before the accumulator is ready, coalesced: lane l loads
+        // granule l % 4 (8 columns) of rows l / 4 + 8 i of the warp's 32 x 32
+        // chunk, 8 rows of 64 bytes per instruction; the chunk is then turned
+        // through its staging buffer so that each lane holds its own row. C is
+        // never the launch's output.
+        constexpr int kChunks = kEpiCols / 32;
         const int crs = lane >> 2, cg = lane & 3;   // coalesced load: sub-row, granule
-        int lt = 0, staged = 0;
+        int lt = 0;
         for (int t = pair; t < n_tiles; t += n_pairs) {
-            const int gi = next.x, b = next.y, m0 = next.z, n0 = next.w;
+            const int gi = next.x, b = next.y, m0 = next.z, n0 = next.w + half * kEpiCols;
             if (t + n_pairs < n_tiles)
                 next = load_tile(tiles + t + n_pairs);
             const GemmGroup &G = L.g[gi];
             const Params p = params[gi];   // in registers: the asm statements below clobber memory
             const int a = lt & 1;
             const int row0 = m0 + (int)rank * BM + q * 32;
-            // C at (row0 + crs, n0 + 8 cg); rows 8 i further for i = 0..3
-            const __nv_bfloat16 *crow =
-                p.c != nullptr ? p.c + (int64_t)b * p.c_bstride + (int64_t)(row0 + crs) * p.ldc +
-                                     n0 + cg * 8
-                               : nullptr;
-            const int64_t c8 = 8 * p.ldc;
-            uint4 cpre[kCPre][4];
-            if (crow != nullptr) {
+            uint4 cpre[kChunks][4];
+            if (p.c != nullptr) {
+                // C at (row0 + crs, n0 + 8 cg); rows 8 i further for i = 0..3
+                const __nv_bfloat16 *crow = p.c + (int64_t)b * p.c_bstride +
+                                            (int64_t)(row0 + crs) * p.ldc + n0 + cg * 8;
 #pragma unroll
-                for (int c = 0; c < kCPre; ++c)
+                for (int c = 0; c < kChunks; ++c)
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
-                        cpre[c][i] = __ldg(reinterpret_cast<const uint4 *>(crow + i * c8 + c * 32));
+                        cpre[c][i] = load_c(crow + 8 * i * p.ldc + c * 32);
             }
             const bool seen = mbar_wait(acc_full(a), (uint32_t)(lt >> 1) & 1u);
             if (!seen)
@@ -549,9 +564,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             // tcgen05.ld is warp-collective: the whole warp goes on, or none of it.
             if (!__all_sync(0xFFFFFFFFu, seen && !*(volatile int *)&aborted))
                 break;
-            const uint32_t acc = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * (int)kTmemCols);
+            const uint32_t acc =
+                tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * (int)kTmemCols + half * kEpiCols);
 #pragma unroll
-            for (int ch = 0; ch < TN / 32; ++ch) {
+            for (int ch = 0; ch < kChunks; ++ch) {
                 uint32_t r[32];
                 tmem_ld32(acc + (uint32_t)(ch * 32), r);
                 float v[32];
@@ -565,23 +581,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                 // and the chunk (its columns share col / TM).
                 const bool mirror = p.sym && row0 / TN < col0 / TM;
                 const bool trans = mirror || p.trans != 0;
-                const uint32_t rb = wbuf + (uint32_t)((staged & 1) * kChunkBytes);
-                const uint32_t tb = rb + (uint32_t)(2 * kChunkBytes);
-                if (lane == 0)   // the buffers' previous group has been read
-                    asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                // Without transposes the two buffers alternate, and only the
+                // chunk before the last one must have been read; a tile's
+                // first chunk may follow one with a transpose.
+                const uint32_t rb = wbuf + (trans ? 0u : (uint32_t)((ch & 1) * kChunkBytes));
+                const uint32_t tb = wbuf + (uint32_t)kChunkBytes;
+                if (lane == 0) {
+                    if (trans || ch == 0)
+                        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                    else
+                        asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                }
                 __syncwarp();
-                if (crow != nullptr) {
+                if (p.c != nullptr) {
                     // the coalesced chunk of C into rb, then this lane's row out
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
-                        const uint4 cv = cpre[ch % kCPre][i];
+                        const uint4 cv = cpre[ch][i];
                         asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
                                      ::"r"(rb + swz64(crs + 8 * i, cg)), "r"(cv.x), "r"(cv.y),
                                        "r"(cv.z), "r"(cv.w)
                                      : "memory");
-                        if (ch + kCPre < TN / 32)   // the slot's next chunk
-                            cpre[ch % kCPre][i] = __ldg(
-                                reinterpret_cast<const uint4 *>(crow + i * c8 + (ch + kCPre) * 32));
                     }
                     __syncwarp();
 #pragma unroll
@@ -629,7 +649,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                         tma_store_3d(mirror ? &G.d : &G.dt, tb, row0, col0, b);
                     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                 }
-                ++staged;
             }
             // this warp's rows of the accumulator are read: release them to
             // the leader's MMA lane
