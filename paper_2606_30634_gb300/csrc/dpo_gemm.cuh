@@ -305,8 +305,11 @@ struct TileGrid {
 // different shapes (the shape groups of a Newton-Schulz step): each group
 // has its own operand and output maps and epilogue, and its tiles follow the
 // previous group's in the launch's order. Small sets then fill the CTA pairs
-// with one launch per product instead of one per shape.
-constexpr int kMaxGroups = 4;
+// with one launch per product instead of one per shape: five odd shapes take
+// 303 us a step on GB300 in one set of launches, 485 us in two (four groups and
+// one). Eight groups are 4.8 KB of launch parameters, of the 32 KB there may
+// be; against four they cost a launch of one group 15 ns.
+constexpr int kMaxGroups = 8;
 
 struct GemmGroup {
     CUtensorMap a, b, d, dt;   // A, B (operands), D and D^T (stores)
@@ -394,11 +397,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             mbar_init(acc_empty(a), 2 * kEpiWarps);   // one arrival per epilogue warp of the pair
         }
         aborted = 0;
-#pragma unroll
-        for (int gi = 0; gi < kMaxGroups; ++gi)
-            params[gi] = L.g[gi].p;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if ((int)threadIdx.x >= 64 && (int)threadIdx.x < 64 + L.n_groups)
+        params[threadIdx.x - 64] = L.g[threadIdx.x - 64].p;
     if (warp == 1) {   // both CTAs of the pair allocate together
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          (uint32_t)__cvta_generic_to_shared(&tmem_slot)),

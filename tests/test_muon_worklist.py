@@ -10,7 +10,7 @@ import numpy as np
 import pytest
 
 from parity_util import TOL_ONE_STEP, TOL_RUN, rel_err
-from test_muon_parity import F, Pair, _flat, close_with_flips
+from test_muon_parity import F, NS_BARS, Pair, _flat, close_with_flips
 
 pytestmark = pytest.mark.gpu
 
@@ -35,5 +35,19 @@ def test_flat_chunks_match_the_oracle(cuda_device, shapes, correction):
             close_with_flips(p.cat(p.gpu.master), _flat(p.ref.x), TOL_RUN, (k + 1) * du, 1e-3)
             close_with_flips(p.cat(p.gpu.ef), _flat(p.ref.u_prev), 1e-5, du, 2e-3)
             close_with_flips(p.cat(p.gpu.stash), _flat(p.ref.stash), TOL_RUN, (k + 1) * du, 1e-3)
+    finally:
+        p.close()
+
+
+def test_more_shape_groups_than_one_launch_takes(cuda_device):
+    """Ten matrix shapes: one GEMM launch takes up to eight, so each product
+    of a Newton-Schulz step is two launches; one step at its normwise and
+    differing-elements bars, and each matrix's output on its own."""
+    p = Pair([(64 + i, 96 + 3 * i) for i in range(10)], cuda_device, ns_steps=1)
+    try:
+        p.step()
+        for g, r in zip(*p.o_pairs()):
+            assert np.linalg.norm(g - r) <= NS_BARS[1][0] * np.linalg.norm(r)
+            assert np.mean(g != r) <= NS_BARS[1][1]
     finally:
         p.close()
