@@ -5,8 +5,9 @@
 //
 // A[b] (M x K) and B[b] (N x K) are row-major bf16 ("K-major" operands), the
 // product accumulates in fp32 in tensor memory, and the epilogue rounds once
-// to bf16. Every dimension is a multiple of the tile (the Newton-Schulz
-// scratch is padded with zeros to multiples of 256), so no tile is partial.
+// to bf16. The Newton-Schulz scratch is padded with zeros to multiples of 256,
+// so every tile is whole; K is taken up to the next multiple of 128, and a
+// tile whose lower or right half is padding skips that half's work.
 //
 // A persistent grid of CTA pairs (clusters of 2, one CTA per SM) walks the
 // 256 x 256 output tiles with the 2-SM MMA. In each CTA:
@@ -219,6 +220,9 @@ __device__ __forceinline__ uint64_t smem_desc_mn(uint32_t addr)
 constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) |
                             ((uint32_t)(TM >> 4) << 24);
 constexpr uint32_t kIdescBmn = kIdesc | (1u << 16);
+// XOR-ed in for N = TN / 2 (a tile whose right half is padding): each CTA of the
+// pair then supplies 64 rows of B.
+constexpr uint32_t kIdescHalfN = ((uint32_t)(TN >> 3) << 17) ^ ((uint32_t)(TN >> 4) << 17);
 
 // One TM x TN x 16 step of the pair, issued by the leader CTA: A rows from
 // both CTAs' shared memory at the descriptor's offset, B likewise, the
@@ -316,12 +320,19 @@ struct GemmGroup {
     Params p;
 };
 
-// The tiles come from a table made at init: x the group, y the batch entry,
-// z and w the tile's first row and column. Each role of the kernel reads its
+// The tiles come from a table made at init: x the group and flags, y the batch
+// entry, z and w the tile's first row and column. kTileHalfM and kTileHalfN
+// mark tiles whose lower or right half lies in the padding of a matrix whose
+// size, rounded up to 128, is an odd multiple of 128: their MMAs take half of
+// the columns, and the CTA of the pair that holds padding rows loads no A and
+// stores nothing. With K rounded up to 128 too, nothing reads what they leave
+// unwritten: it stays the zeros of init, which a computed tile would write. Each role of the kernel reads its
 // pair's next entry while it works on the current one. Deriving them from t
 // in the kernel (a search over the groups, four divisions) read the launch's
 // parameters through dependent loads and took every role, the MMA lane among
 // them, some 3,900 cycles per tile: a third of a K = 768 tile's time.
+constexpr int kTileGroup = 0xff, kTileHalfM = 0x100, kTileHalfN = 0x200;
+
 struct GemmLaunch {
     GemmGroup g[kMaxGroups];
     const int4 *tiles;
@@ -429,12 +440,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             }
             int it = 0;   // k-blocks issued by this CTA
             for (int t = pair; t < n_tiles && !*(volatile int *)&aborted; t += n_pairs) {
-                const int gi = next.x, b = next.y, m0 = next.z, n0 = next.w;
+                const int gi = next.x & kTileGroup, b = next.y, m0 = next.z, n0 = next.w;
+                const bool half_m = next.x & kTileHalfM, half_n = next.x & kTileHalfN;
                 if (t + n_pairs < n_tiles)
                     next = load_tile(tiles + t + n_pairs);
+                // both CTAs' bytes of a stage: A of the rows that are not all
+                // padding; of a half-wide MN-major B one box of 64 columns, of
+                // a K-major one the box of 128 rows of which 64 are used
+                const uint32_t bytes = (uint32_t)((half_m ? 1 : 2) * kABytes +
+                                                  (BMN && half_n ? 1 : 2) * kBBytes);
+                const bool load_a = leader || !half_m;
                 const CUtensorMap *tma_a = &L.g[gi].a, *tma_b = &L.g[gi].b;
                 const int kb_n = params[gi].k_blocks;
-                const int ma = m0 + (int)rank * BM, nb_ = n0 + (int)rank * BH;
+                const int ma = m0 + (int)rank * BM, nb_ = n0 + (int)rank * (half_n ? BH / 2 : BH);
                 for (int kb = 0; kb < kb_n; ++kb, ++it) {
                     const int s = it % kStages;
                     const uint32_t ph = (uint32_t)(it / kStages) & 1u;
@@ -445,16 +463,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                     }
                     const uint32_t fbar = map_to_rank(full(s), 0);
                     if (leader)   // the leader's barrier counts both CTAs' bytes
-                        mbar_arrive_expect_tx(full(s), (uint32_t)(2 * kStageBytes));
+                        mbar_arrive_expect_tx(full(s), bytes);
 #pragma unroll
                     for (int h = 0; h < BK / kBoxK; ++h) {   // the two 64-wide K halves
                         const int k0 = kb * BK + h * kBoxK;
                         const uint32_t ah = sa + (uint32_t)(s * kABytes + h * (kABytes / 2));
                         const uint32_t bh = sb + (uint32_t)(s * kBBytes + h * (kBBytes / 2));
-                        tma_load_3d(ah, tma_a, k0, ma, b, fbar);
+                        if (load_a)
+                            tma_load_3d(ah, tma_a, k0, ma, b, fbar);
                         if (BMN) {   // two 64 x 64 boxes: N columns nb_.. and nb_ + 64..
                             tma_load_3d(bh, tma_b, nb_, k0, b, fbar);
-                            tma_load_3d(bh + (uint32_t)(kBBytes / 4), tma_b, nb_ + 64, k0, b, fbar);
+                            if (!half_n)
+                                tma_load_3d(bh + (uint32_t)(kBBytes / 4), tma_b, nb_ + 64, k0, b,
+                                            fbar);
                         } else {
                             tma_load_3d(bh, tma_b, k0, nb_, b, fbar);
                         }
@@ -473,7 +494,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         if (lane == 0 && leader) {
             int it = 0, lt = 0;   // k-blocks consumed, tiles accumulated
             for (int t = pair; t < n_tiles && !*(volatile int *)&aborted; t += n_pairs) {
-                const int kb_n = params[next.x].k_blocks;
+                const int kb_n = params[next.x & kTileGroup].k_blocks;
+                const uint32_t idesc =
+                    (BMN ? kIdescBmn : kIdesc) ^ (next.x & kTileHalfN ? kIdescHalfN : 0u);
                 if (t + n_pairs < n_tiles)
                     next = load_tile(tiles + t + n_pairs);
                 const int a = lt & 1;
@@ -504,7 +527,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                         const uint64_t ad = smem_desc(ah + (uint32_t)(kk * 32));
                         const uint64_t bd = BMN ? smem_desc_mn(bh + (uint32_t)(kk * 16 * 128))
                                                 : smem_desc(bh + (uint32_t)(kk * 32));
-                        mma_bf16(d, ad, bd, BMN ? kIdescBmn : kIdesc, (kb | k) != 0 ? 1u : 0u);
+                        mma_bf16(d, ad, bd, idesc, (kb | k) != 0 ? 1u : 0u);
                     }
                     mma_commit_pair(empty(s));
                 }
@@ -541,7 +564,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const int crs = lane >> 2, cg = lane & 3;   // coalesced load: sub-row, granule
         int lt = 0;
         for (int t = pair; t < n_tiles; t += n_pairs) {
-            const int gi = next.x, b = next.y, m0 = next.z, n0 = next.w + half * kEpiCols;
+            const int gi = next.x & kTileGroup, b = next.y, m0 = next.z;
+            const int n0 = next.w + half * kEpiCols;
+            // this warp's rows or columns are all padding: it only passes the
+            // accumulator on
+            const bool idle = (next.x & kTileHalfM && !leader) || (next.x & kTileHalfN && half);
             if (t + n_pairs < n_tiles)
                 next = load_tile(tiles + t + n_pairs);
             const GemmGroup &G = L.g[gi];
@@ -549,7 +576,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             const int a = lt & 1;
             const int row0 = m0 + (int)rank * BM + q * 32;
             uint4 cpre[kChunks][4];
-            if (p.c != nullptr) {
+            if (p.c != nullptr && !idle) {
                 // C at (row0 + crs, n0 + 8 cg); rows 8 i further for i = 0..3
                 const __nv_bfloat16 *crow = p.c + (int64_t)b * p.c_bstride +
                                             (int64_t)(row0 + crs) * p.ldc + n0 + cg * 8;
@@ -568,6 +595,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                 break;
             const uint32_t acc =
                 tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * (int)kTmemCols + half * kEpiCols);
+            if (!idle)
 #pragma unroll
             for (int ch = 0; ch < kChunks; ++ch) {
                 uint32_t r[32];

@@ -883,7 +883,7 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
             auto &p = ls.prod[prod];
             auto k_of = [&](int q) {
                 const Group &g = c->groups[ls.group[q]];
-                return prod == 0 ? g.W : g.R;
+                return prod == 0 ? g.w : g.r;
             };
             for (int q = 0; q < ls.n; ++q)
                 p.order[q] = q;
@@ -894,7 +894,12 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
                 const dpo::gemm::TileGrid tg{(int)(g.R / dpo::gemm::TM),
                                              (int)((prod == 2 ? g.W : g.R) / dpo::gemm::TN),
                                              (int)g.mats.size(), prod != 2};
-                tg.walk([&](int b, int m0, int n0) { tiles.push_back(make_int4(q, b, m0, n0)); });
+                const int64_t rows = g.r, cols = prod == 2 ? g.w : g.r;
+                tg.walk([&](int b, int m0, int n0) {
+                    const int flags = (rows <= m0 + dpo::gemm::TM / 2 ? dpo::gemm::kTileHalfM : 0) |
+                                      (cols <= n0 + dpo::gemm::TN / 2 ? dpo::gemm::kTileHalfN : 0);
+                    tiles.push_back(make_int4(q | flags, b, m0, n0));
+                });
             }
             p.tiles = (int)((int64_t)tiles.size() - p.first);
         }
@@ -1214,7 +1219,7 @@ int orthogonalize(dpo_muon_ctx *c, cudaStream_t s, bool predict)
                 p.err = c->d_err;
                 // A = X X^T
                 p.alpha = 1.0f;
-                p.k_blocks = (int)(g.W / dpo::gemm::BK);
+                p.k_blocks = (int)((g.w + dpo::gemm::BK - 1) / dpo::gemm::BK);
                 p.sym = 1;
                 p.stall = st_xx;
                 xx[q] = GemmJob{&g.x128[cur], &g.x128[cur], &g.st_a, &g.st_a, p};
@@ -1224,7 +1229,7 @@ int orthogonalize(dpo_muon_ctx *c, cudaStream_t s, bool predict)
                 p.c_bstride = g.R * g.R;
                 p.alpha = c->hp.ns_c;
                 p.beta = c->hp.ns_b;
-                p.k_blocks = (int)(g.R / dpo::gemm::BK);
+                p.k_blocks = (int)((g.r + dpo::gemm::BK - 1) / dpo::gemm::BK);
                 p.stall = st_aa;
                 aa[q] = GemmJob{&g.a128, &g.a128, &g.st_b, &g.st_b, p};
                 // X <- B X + a X (X read MN-major in place of X^T), and at the
@@ -1236,7 +1241,7 @@ int orthogonalize(dpo_muon_ctx *c, cudaStream_t s, bool predict)
                 p.c_bstride = g.R * g.W;
                 p.alpha = 1.0f;
                 p.beta = c->hp.ns_a;
-                p.k_blocks = (int)(g.R / dpo::gemm::BK);
+                p.k_blocks = (int)((g.r + dpo::gemm::BK - 1) / dpo::gemm::BK);
                 p.stall = st_bx;
                 bx[q] = GemmJob{&g.b128, &g.x_mn[cur], &g.st_x[nxt], &g.st_xt, p};
             }

@@ -51,3 +51,24 @@ def test_more_shape_groups_than_one_launch_takes(cuda_device):
             assert np.mean(g != r) <= NS_BARS[1][1]
     finally:
         p.close()
+
+
+# sizes on either side of a tile's half (128) and whole (256), in both dimensions
+HALVES = [(127, 129), (128, 128), (129, 384), (256, 385), (257, 640), (384, 257), (385, 513),
+          (512, 641), (640, 640)]
+
+
+@pytest.mark.parametrize("steps", [1, 2])
+def test_tiles_half_in_the_padding(cuda_device, steps):
+    """Matrices whose last tiles are half padding, wide and tall, over two
+    calls (the second reads scratch that the first left): normwise and
+    differing elements of each Newton-Schulz output at the bars of its steps."""
+    p = Pair(HALVES, cuda_device, ns_steps=steps)
+    try:
+        for _ in range(2):
+            p.step()
+            for shape, g, r in zip(HALVES, *p.o_pairs()):
+                assert np.linalg.norm(g - r) <= NS_BARS[steps][0] * np.linalg.norm(r), shape
+                assert np.mean(g != r) <= NS_BARS[steps][1], shape
+    finally:
+        p.close()
