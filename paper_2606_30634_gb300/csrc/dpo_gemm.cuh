@@ -10,7 +10,9 @@
 // tile whose lower or right half is padding skips that half's work.
 //
 // A persistent grid of CTA pairs (clusters of 2, one CTA per SM) walks the
-// 256 x 256 output tiles with the 2-SM MMA. In each CTA:
+// 256 x 256 output tiles with the 2-SM MMA; launches of few tiles take the
+// same kernel by single CTAs instead (128 x 128 tiles, the 1-SM MMA, no
+// cluster; CG = 1), where "both CTAs" below is the one. In each CTA:
 //   warp 0      TMA producer: this CTA's 128 x 128 half of the A block and
 //               128 x 128 half of the B block (bf16, 128-byte swizzle, two
 //               64-wide boxes each) into a 3-stage ring, completing on the
@@ -52,7 +54,11 @@ namespace gemm {
 // spans BK = 128 of K as two TMA boxes of kBoxK = 64 (the 128-byte swizzle
 // span); eight MMAs per stage halve the barrier hand-offs per MMA against
 // 64-wide stages, which measured 10% faster on GB300 at equal ring size.
-constexpr int TM = 256, TN = 256, BM = 128, BH = 128, BK = 128, kBoxK = 64, kStages = 3;
+// kTile(2) is that tile. kTile(1) is the tile of a single CTA (128 x 128, the
+// 1-SM MMA, the same stages), for launches of few tiles.
+__host__ __device__ constexpr int kTile(int cg) { return 128 * cg; }
+constexpr int TM = kTile(2), TN = kTile(2);
+constexpr int BM = 128, BH = 128, BK = 128, kBoxK = 64, kStages = 3;
 // Epilogue warps: two per TMEM lane quarter, each taking half of the tile's
 // columns: a tile's epilogue is a serial chain per warp (TMEM read, addend,
 // staging, store), which the 6 k-blocks of a K = 768 tile do not hide at four
@@ -61,8 +67,6 @@ constexpr int TM = 256, TN = 256, BM = 128, BH = 128, BK = 128, kBoxK = 64, kSta
 // layer, whose tiles have 32 k-blocks, is unchanged.
 constexpr int kEpiWarps = 8;
 constexpr int kThreads = 64 + 32 * kEpiWarps;
-constexpr int kEpiCols = TN * 4 / kEpiWarps;   // columns per epilogue warp
-constexpr uint32_t kTmemCols = 256;                  // one accumulator (fp32, TN columns)
 constexpr int kABytes = BM * BK * 2;                 // 32 KiB
 constexpr int kBBytes = BH * BK * 2;                 // 32 KiB
 constexpr int kStageBytes = kABytes + kBBytes;       // 64 KiB per CTA
@@ -136,16 +140,24 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t byt
                  : "memory");
 }
 
-// TMA tile load into this CTA's shared memory; the mbarrier (a shared::cluster
-// address) may belong to either CTA of the pair.
+// TMA tile load into this CTA's shared memory; with CG == 2 the mbarrier (a
+// shared::cluster address) may belong to either CTA of the pair.
+template <int CG>
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, int x, int y,
                                             int z, uint32_t bar_cluster)
 {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar_cluster)
-        : "memory");
+    if (CG == 2)
+        asm volatile(
+            "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+            " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+            "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar_cluster)
+            : "memory");
+    else
+        asm volatile(
+            "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
+            " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+            "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar_cluster)
+            : "memory");
 }
 
 // TMA store of a 32 x 32 bf16 box from this CTA's shared memory to global
@@ -181,16 +193,26 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank)
     return r;
 }
 
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster)
+// One arrival on the leader's mbarrier at this shared::cta offset.
+template <int CG> __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster)
-                 : "memory");
+    if (CG == 2)
+        asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(
+                         map_to_rank(bar, 0))
+                     : "memory");
+    else
+        asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-__device__ __forceinline__ void cluster_sync()
+// All threads of the CTA, or of the pair.
+template <int CG> __device__ __forceinline__ void group_sync()
 {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (CG == 2) {
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    } else {
+        __syncthreads();
+    }
 }
 
 // Shared-memory matrix descriptor of a K-major operand tile stored as rows of
@@ -215,36 +237,79 @@ __device__ __forceinline__ uint64_t smem_desc_mn(uint32_t addr)
 }
 
 // Instruction descriptor of kind::f16: fp32 accumulator, bf16 A and B, A
-// K-major, N = TN, M = TM (the pair's 2-SM shape); B K-major, or MN-major
-// with bit 16 (B read as stored row-major along N).
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) |
-                            ((uint32_t)(TM >> 4) << 24);
-constexpr uint32_t kIdescBmn = kIdesc | (1u << 16);
+// K-major, N = M = kTile(cg) (cg 2: the pair's 2-SM shape); B K-major, or
+// MN-major with bit 16 (B read as stored row-major along N).
+__host__ __device__ constexpr uint32_t idesc_of(int cg, bool bmn)
+{
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTile(cg) >> 3) << 17) |
+           ((uint32_t)(kTile(cg) >> 4) << 24) | (bmn ? 1u << 16 : 0u);
+}
 // XOR-ed in for N = TN / 2 (a tile whose right half is padding): each CTA of the
 // pair then supplies 64 rows of B.
 constexpr uint32_t kIdescHalfN = ((uint32_t)(TN >> 3) << 17) ^ ((uint32_t)(TN >> 4) << 17);
 
-// One TM x TN x 16 step of the pair, issued by the leader CTA: A rows from
+// One 16-deep step of a tile, issued by the leader CTA; CG == 2: A rows from
 // both CTAs' shared memory at the descriptor's offset, B likewise, the
 // accumulator rows in each CTA's TMEM.
+template <int CG>
 __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a_desc, uint64_t b_desc,
                                          uint32_t idesc, uint32_t accumulate)
 {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate));
+    if (CG == 2)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+            "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate));
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+            "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate));
 }
 
-// Arrive on the mbarrier at this shared::cta offset in both CTAs of the pair
+// Arrive on the mbarrier at this shared::cta offset, in both CTAs of a pair,
 // once the leader's MMAs issued so far have completed.
-__device__ __forceinline__ void mma_commit_pair(uint32_t bar)
+template <int CG> __device__ __forceinline__ void mma_commit(uint32_t bar)
 {
-    asm volatile(
-        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
-        " [%0], %1;" ::"r"(bar), "h"((uint16_t)0x3)
-        : "memory");
+    if (CG == 2)
+        asm volatile(
+            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
+            " [%0], %1;" ::"r"(bar), "h"((uint16_t)0x3)
+            : "memory");
+    else
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                     ::"r"(bar) : "memory");
+}
+
+// TMEM columns of both accumulators, allocated and freed by one warp (of both
+// CTAs of a pair).
+template <int CG> __device__ __forceinline__ void tmem_alloc(uint32_t slot)
+{
+    if (CG == 2) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot),
+                     "r"(2 * kTile(CG))
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot),
+                     "r"(2 * kTile(CG))
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+}
+
+template <int CG> __device__ __forceinline__ void tmem_free(uint32_t tmem)
+{
+    if (CG == 2)
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                     "r"(2 * kTile(CG))
+                     : "memory");
+    else
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                     "r"(2 * kTile(CG))
+                     : "memory");
 }
 
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
@@ -280,10 +345,10 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
 // of them), so the pairs' shares of its work differ by at most one tile, and
 // the tiles in flight at once read the first block rows of the operand before
 // the pairs move on to the last ones.
-constexpr int kBandRows = 16;   // block rows per band of a full product's walk
+constexpr int kBandRows = 16;   // block rows per band of a full product's walk (256-row tiles)
 
 struct TileGrid {
-    int m_tiles, n_tiles, nb, sym;
+    int m_tiles, n_tiles, nb, sym, tile;
     int per_batch() const { return sym ? m_tiles * (m_tiles + 1) / 2 : m_tiles * n_tiles; }
     int count() const { return per_batch() * nb; }
     // fn(batch entry, first row, first column) for every tile in order
@@ -294,12 +359,12 @@ struct TileGrid {
             if (sym) {
                 for (int n = 0; n < n_tiles; ++n)
                     for (int m = 0; m <= n; ++m)
-                        fn(b, m * TM, n * TN);
+                        fn(b, m * tile, n * tile);
             } else {
                 for (int first = 0; first < m_tiles; first += kBandRows)
                     for (int n = 0; n < n_tiles; ++n)
                         for (int m = first; m < m_tiles && m < first + kBandRows; ++m)
-                            fn(b, m * TM, n * TN);
+                            fn(b, m * tile, n * tile);
             }
         }
     }
@@ -326,8 +391,13 @@ struct GemmGroup {
 // size, rounded up to 128, is an odd multiple of 128: their MMAs take half of
 // the columns, and the CTA of the pair that holds padding rows loads no A and
 // stores nothing. With K rounded up to 128 too, nothing reads what they leave
-// unwritten: it stays the zeros of init, which a computed tile would write. Each role of the kernel reads its
-// pair's next entry while it works on the current one. Deriving them from t
+// unwritten: it stays the zeros of init, which a computed tile would write.
+// GB300, without against with the halves and the rounded K, whole step: four
+// 384-wide layers 231 -> 207 us, three 640-wide ones 343 -> 329, two 1100-wide
+// ones 735 -> 702; where no tile has a padded half it costs up to 1 % (two
+// 256x768 matrices 132.0 -> 133.4, GPT-2 1789 -> 1793).
+// Each role of the kernel reads its next entry while it works on the current
+// one. Deriving them from t
 // in the kernel (a search over the groups, four divisions) read the launch's
 // parameters through dependent loads and took every role, the MMA lane among
 // them, some 3,900 cycles per tile: a third of a K = 768 tile's time.
@@ -373,10 +443,12 @@ __device__ __forceinline__ int4 load_tile(const int4 *p)
 //   acc_empty[a] (leader) all epilogue warps of the pair have read it
 // BMN: the B operand is stored N-contiguous (a row-major K x N matrix) and
 // loaded as two 64 x 64 boxes per stage, read MN-major by the MMA.
-template <bool BMN>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+template <bool BMN, int CG>
+__global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
     ns_gemm_kernel(const __grid_constant__ GemmLaunch L)
 {
+    constexpr int T = kTile(CG);                   // tile side, TMEM columns of an accumulator
+    constexpr int kEpiCols = T * 4 / kEpiWarps;    // columns per epilogue warp
     unsigned int *const err = L.g[0].p.err;   // err and stall are the launch's
     const int stall = L.g[0].p.stall;
     extern __shared__ uint8_t smem_raw[];
@@ -386,9 +458,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     __shared__ Params params[kMaxGroups];   // read per tile, by every role
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = cluster_rank();
+    const uint32_t rank = CG == 2 ? cluster_rank() : 0u;
     const bool leader = rank == 0;
-    const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+    const int pair = blockIdx.x / CG, n_pairs = gridDim.x / CG;
     const uint32_t raw = (uint32_t)__cvta_generic_to_shared(smem_raw);
     const uint32_t ring = (raw + 1023u) & ~1023u;   // the swizzle atoms repeat every 1024 B
     const uint32_t sa = ring, sb = ring + kStages * kABytes;
@@ -405,22 +477,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(acc_full(a), 1);
-            mbar_init(acc_empty(a), 2 * kEpiWarps);   // one arrival per epilogue warp of the pair
+            mbar_init(acc_empty(a), CG * kEpiWarps);   // one arrival per epilogue warp of the pair
         }
         aborted = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if ((int)threadIdx.x >= 64 && (int)threadIdx.x < 64 + L.n_groups)
         params[threadIdx.x - 64] = L.g[threadIdx.x - 64].p;
-    if (warp == 1) {   // both CTAs of the pair allocate together
-        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                         (uint32_t)__cvta_generic_to_shared(&tmem_slot)),
-                     "r"(2 * kTmemCols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-    }
+    if (warp == 1)   // both CTAs of a pair allocate together
+        tmem_alloc<CG>((uint32_t)__cvta_generic_to_shared(&tmem_slot));
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    cluster_sync();   // barriers of both CTAs initialised before any remote use
+    group_sync<CG>();   // barriers of both CTAs initialised before any remote use
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
     const int n_tiles = L.n_tiles;
@@ -441,14 +508,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             int it = 0;   // k-blocks issued by this CTA
             for (int t = pair; t < n_tiles && !*(volatile int *)&aborted; t += n_pairs) {
                 const int gi = next.x & kTileGroup, b = next.y, m0 = next.z, n0 = next.w;
-                const bool half_m = next.x & kTileHalfM, half_n = next.x & kTileHalfN;
+                const bool half_m = CG == 2 && (next.x & kTileHalfM);
+                const bool half_n = CG == 2 && (next.x & kTileHalfN);
                 if (t + n_pairs < n_tiles)
                     next = load_tile(tiles + t + n_pairs);
                 // both CTAs' bytes of a stage: A of the rows that are not all
                 // padding; of a half-wide MN-major B one box of 64 columns, of
                 // a K-major one the box of 128 rows of which 64 are used
-                const uint32_t bytes = (uint32_t)((half_m ? 1 : 2) * kABytes +
-                                                  (BMN && half_n ? 1 : 2) * kBBytes);
+                const uint32_t bytes =
+                    CG == 1 ? (uint32_t)kStageBytes
+                            : (uint32_t)((half_m ? 1 : 2) * kABytes +
+                                         (BMN && half_n ? 1 : 2) * kBBytes);
                 const bool load_a = leader || !half_m;
                 const CUtensorMap *tma_a = &L.g[gi].a, *tma_b = &L.g[gi].b;
                 const int kb_n = params[gi].k_blocks;
@@ -461,7 +531,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                         aborted = 1;
                         break;
                     }
-                    const uint32_t fbar = map_to_rank(full(s), 0);
+                    const uint32_t fbar = CG == 2 ? map_to_rank(full(s), 0) : full(s);
                     if (leader)   // the leader's barrier counts both CTAs' bytes
                         mbar_arrive_expect_tx(full(s), bytes);
 #pragma unroll
@@ -470,14 +540,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                         const uint32_t ah = sa + (uint32_t)(s * kABytes + h * (kABytes / 2));
                         const uint32_t bh = sb + (uint32_t)(s * kBBytes + h * (kBBytes / 2));
                         if (load_a)
-                            tma_load_3d(ah, tma_a, k0, ma, b, fbar);
+                            tma_load_3d<CG>(ah, tma_a, k0, ma, b, fbar);
                         if (BMN) {   // two 64 x 64 boxes: N columns nb_.. and nb_ + 64..
-                            tma_load_3d(bh, tma_b, nb_, k0, b, fbar);
+                            tma_load_3d<CG>(bh, tma_b, nb_, k0, b, fbar);
                             if (!half_n)
-                                tma_load_3d(bh + (uint32_t)(kBBytes / 4), tma_b, nb_ + 64, k0, b,
-                                            fbar);
+                                tma_load_3d<CG>(bh + (uint32_t)(kBBytes / 4), tma_b, nb_ + 64, k0,
+                                                b, fbar);
                         } else {
-                            tma_load_3d(bh, tma_b, k0, nb_, b, fbar);
+                            tma_load_3d<CG>(bh, tma_b, k0, nb_, b, fbar);
                         }
                     }
                 }
@@ -496,7 +566,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             for (int t = pair; t < n_tiles && !*(volatile int *)&aborted; t += n_pairs) {
                 const int kb_n = params[next.x & kTileGroup].k_blocks;
                 const uint32_t idesc =
-                    (BMN ? kIdescBmn : kIdesc) ^ (next.x & kTileHalfN ? kIdescHalfN : 0u);
+                    idesc_of(CG, BMN) ^ (CG == 2 && (next.x & kTileHalfN) ? kIdescHalfN : 0u);
                 if (t + n_pairs < n_tiles)
                     next = load_tile(tiles + t + n_pairs);
                 const int a = lt & 1;
@@ -507,7 +577,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t d = tmem + (uint32_t)(a * (int)kTmemCols);
+                const uint32_t d = tmem + (uint32_t)(a * T);
                 bool ok = true;
                 for (int kb = 0; kb < kb_n; ++kb, ++it) {
                     const int s = it % kStages;
@@ -527,11 +597,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                         const uint64_t ad = smem_desc(ah + (uint32_t)(kk * 32));
                         const uint64_t bd = BMN ? smem_desc_mn(bh + (uint32_t)(kk * 16 * 128))
                                                 : smem_desc(bh + (uint32_t)(kk * 32));
-                        mma_bf16(d, ad, bd, idesc, (kb | k) != 0 ? 1u : 0u);
+                        mma_bf16<CG>(d, ad, bd, idesc, (kb | k) != 0 ? 1u : 0u);
                     }
-                    mma_commit_pair(empty(s));
+                    mma_commit<CG>(empty(s));
                 }
-                mma_commit_pair(acc_full(a));   // when this tile's MMAs have completed
+                mma_commit<CG>(acc_full(a));   // when this tile's MMAs have completed
                 ++lt;
                 if (!ok) {
                     // the MMAs issued for this tile finish before the pair
@@ -568,7 +638,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             const int n0 = next.w + half * kEpiCols;
             // this warp's rows or columns are all padding: it only passes the
             // accumulator on
-            const bool idle = (next.x & kTileHalfM && !leader) || (next.x & kTileHalfN && half);
+            const bool idle = CG == 2 && ((next.x & kTileHalfM && !leader) ||
+                                          (next.x & kTileHalfN && half));
             if (t + n_pairs < n_tiles)
                 next = load_tile(tiles + t + n_pairs);
             const GemmGroup &G = L.g[gi];
@@ -594,7 +665,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             if (!__all_sync(0xFFFFFFFFu, seen && !*(volatile int *)&aborted))
                 break;
             const uint32_t acc =
-                tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * (int)kTmemCols + half * kEpiCols);
+                tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * T + half * kEpiCols);
             if (!idle)
 #pragma unroll
             for (int ch = 0; ch < kChunks; ++ch) {
@@ -606,10 +677,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                     v[j] = p.alpha * __uint_as_float(r[j]);
                 const int col0 = n0 + ch * 32;
                 // Mirror of a symmetric product: (col, row) lies in the tile
-                // (col / TM, row / TN), not computed when row / TN < col / TM
-                // (TM == TN). Uniform over the warp (its rows share row / TN)
-                // and the chunk (its columns share col / TM).
-                const bool mirror = p.sym && row0 / TN < col0 / TM;
+                // (col / T, row / T), not computed when row / T < col / T.
+                // Uniform over the warp (its rows share row / T) and the chunk
+                // (its columns share col / T).
+                const bool mirror = p.sym && row0 / T < col0 / T;
                 const bool trans = mirror || p.trans != 0;
                 // Without transposes the two buffers alternate, and only the
                 // chunk before the last one must have been read; a tile's
@@ -685,7 +756,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0)
-                mbar_arrive_cluster(map_to_rank(acc_empty(a), 0));
+                mbar_arrive<CG>(acc_empty(a));
             ++lt;
         }
         if (lane == 0)   // every store has been written before the CTA ends
@@ -694,12 +765,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     }
     __syncthreads();
-    cluster_sync();   // no CTA leaves while its peer may still read its shared memory
+    if (CG == 2)
+        group_sync<CG>();   // no CTA leaves while its peer may still read its shared memory
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                     "r"(2 * kTmemCols)
-                     : "memory");
+        tmem_free<CG>(tmem);
     }
 }
 

@@ -567,6 +567,44 @@ bool make_store_map(CUtensorMap *m, void *base, int64_t rows, int64_t cols, int6
                CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+using GemmFn = void (*)(dpo::gemm::GemmLaunch);
+
+GemmFn gemm_kernel(bool b_mn, int cg)
+{
+    if (cg == 2)
+        return b_mn ? dpo::gemm::ns_gemm_kernel<true, 2> : dpo::gemm::ns_gemm_kernel<false, 2>;
+    return b_mn ? dpo::gemm::ns_gemm_kernel<true, 1> : dpo::gemm::ns_gemm_kernel<false, 1>;
+}
+
+// Estimated clocks of a launch over tiles with these K blocks, dealt round-robin
+// to `slots` CTAs (cg 1) or pairs (cg 2): a slot's mainloops run back to back,
+// each hiding the epilogue of the tile before it, and the last epilogue shows.
+// Each product of a launch set takes the form with the smaller estimate. The
+// single CTA's tile needs as many bytes per K block as its half of a pair's
+// and does half of the multiplications, so it loses once every SM has several
+// tiles; with few it spreads a product over more SMs, computes less past the
+// diagonal and has half the epilogue. GB300, whole step, all products by pairs
+// / by single CTAs / by this rule: two 256x768 matrices 133 / 99 / 99 us, one
+// 768-wide layer 289 / 243 / 243, three of them 466 / 480 / 464, two
+// 1024-wide layers 627 / 604 / 604, a 1536-wide one 809 / 861 / 808, an
+// 1100-wide one 405 / 410 / 409. The clocks per K block and per epilogue are
+// the set, of nine tried, that came closest to the better form on 15 sets.
+int64_t launch_clocks(const std::vector<int> &k_blocks, int slots, int cg)
+{
+    const int64_t block = cg == 1 ? 700 : 1100, epilogue = cg == 1 ? 2600 : 5000;
+    int64_t worst = 0;
+    for (int s = 0; s < slots && s < (int)k_blocks.size(); ++s) {
+        int64_t t = 0;
+        for (size_t i = s; i < k_blocks.size(); i += slots)
+            t += std::max(k_blocks[i] * block, i == (size_t)s ? (int64_t)0 : epilogue);
+        worst = std::max(worst, t + epilogue);
+    }
+    return worst;
+}
+
+// Rounds of single-CTA tiles above which a launch goes to the pairs unweighed.
+constexpr int64_t kFewRounds = 4;
+
 int64_t pad_up(int64_t v) { return (v + kPad - 1) / kPad * kPad; }
 
 // One Newton-Schulz launch set: up to kMaxGroups shape groups that share each
@@ -579,6 +617,7 @@ struct LaunchSet {
         int order[dpo::gemm::kMaxGroups];   // positions in group[]
         int64_t first = 0;                  // first entry of the tile table
         int tiles = 0;
+        int cg = 2;                         // CTAs per tile: 256 x 256 pairs, or 128 x 128
     } prod[3];
 };
 
@@ -614,6 +653,7 @@ struct dpo_muon_ctx {
     dpo::muon::ApplyScalars *d_asc = nullptr;
     int sms = 0;
     int gemm_pairs = 0;   // clusters of 2 the GEMM kernel keeps resident at once
+    int gemm_ctas = 0;    // CTAs of its single-CTA form
     int stall_launches = 0;   // dpo_muon_test_stall: GEMM launches left to stall
     std::vector<dpo_matrix> mats;
     std::vector<DevMat> host_mats;
@@ -835,26 +875,27 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
             g.has_tall = g.has_tall || mats[mi].rows > mats[mi].cols;
     }
     c->ws_bytes = ws;
-    // CTA pairs the GEMM kernels keep resident at once (a failure is reported
-    // after the allocations, where the launches it stops would come).
-    c->gemm_pairs = 1 << 30;
+    // CTA pairs and single CTAs the GEMM kernels keep resident at once (a
+    // failure is reported after the allocations, where the launches it stops
+    // would come).
+    c->gemm_pairs = c->gemm_ctas = 1 << 30;
     cudaError_t e_gemm = cudaSuccess;
-    for (const void *fn : {(const void *)dpo::gemm::ns_gemm_kernel<false>,
-                           (const void *)dpo::gemm::ns_gemm_kernel<true>}) {
-        e_gemm = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      dpo::gemm::kSmemBytes);
-        int pairs = 0;
-        if (e_gemm == cudaSuccess) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(2 * std::max(1, c->sms / 2));
-            cfg.blockDim = dim3(dpo::gemm::kThreads);
-            cfg.dynamicSmemBytes = dpo::gemm::kSmemBytes;
-            e_gemm = cudaOccupancyMaxActiveClusters(&pairs, fn, &cfg);
+    for (int cg = 1; cg <= 2 && e_gemm == cudaSuccess; ++cg)
+        for (int mn = 0; mn < 2 && e_gemm == cudaSuccess; ++mn) {
+            const void *fn = (const void *)gemm_kernel(mn != 0, cg);
+            e_gemm = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          dpo::gemm::kSmemBytes);
+            int n_res = 0;
+            if (e_gemm == cudaSuccess) {
+                cudaLaunchConfig_t cfg = {};
+                cfg.gridDim = dim3(2 * std::max(1, c->sms / 2));
+                cfg.blockDim = dim3(dpo::gemm::kThreads);
+                cfg.dynamicSmemBytes = dpo::gemm::kSmemBytes;
+                e_gemm = cudaOccupancyMaxActiveClusters(&n_res, fn, &cfg);
+            }
+            int &have = cg == 2 ? c->gemm_pairs : c->gemm_ctas;
+            have = std::min(have, n_res);
         }
-        if (e_gemm != cudaSuccess)
-            break;
-        c->gemm_pairs = std::min(c->gemm_pairs, pairs);
-    }
     // When some shape group's launches are short (at most 16 rounds of tiles
     // over the CTA pairs), each product of a Newton-Schulz step covers all
     // shape groups in one launch: one group's tiles fill the pairs another
@@ -888,20 +929,39 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
             for (int q = 0; q < ls.n; ++q)
                 p.order[q] = q;
             std::stable_sort(p.order, p.order + ls.n, [&](int x, int y) { return k_of(x) > k_of(y); });
-            p.first = (int64_t)tiles.size();
-            for (int q = 0; q < ls.n; ++q) {
-                const Group &g = c->groups[ls.group[p.order[q]]];
-                const dpo::gemm::TileGrid tg{(int)(g.R / dpo::gemm::TM),
-                                             (int)((prod == 2 ? g.W : g.R) / dpo::gemm::TN),
-                                             (int)g.mats.size(), prod != 2};
-                const int64_t rows = g.r, cols = prod == 2 ? g.w : g.r;
-                tg.walk([&](int b, int m0, int n0) {
-                    const int flags = (rows <= m0 + dpo::gemm::TM / 2 ? dpo::gemm::kTileHalfM : 0) |
-                                      (cols <= n0 + dpo::gemm::TN / 2 ? dpo::gemm::kTileHalfN : 0);
-                    tiles.push_back(make_int4(q | flags, b, m0, n0));
-                });
+            std::vector<int4> list[2];   // by single CTAs, by pairs
+            std::vector<int> k_blocks[2];
+            for (int cg = 1; cg <= 2; ++cg) {
+                const int side = dpo::gemm::kTile(cg);
+                for (int q = 0; q < ls.n; ++q) {
+                    const Group &g = c->groups[ls.group[p.order[q]]];
+                    const int64_t rows = g.r, cols = prod == 2 ? g.w : g.r;
+                    const dpo::gemm::TileGrid tg{(int)((rows + side - 1) / side),
+                                                 (int)((cols + side - 1) / side),
+                                                 (int)g.mats.size(), prod != 2, side};
+                    if (cg == 1 && tg.count() + (int64_t)list[0].size() >
+                                       kFewRounds * c->gemm_ctas) {
+                        list[0].clear();
+                        break;
+                    }
+                    const int kb = (int)((k_of(p.order[q]) + dpo::gemm::BK - 1) / dpo::gemm::BK);
+                    tg.walk([&](int b, int m0, int n0) {
+                        int flags = 0;
+                        if (cg == 2)
+                            flags = (rows <= m0 + side / 2 ? dpo::gemm::kTileHalfM : 0) |
+                                    (cols <= n0 + side / 2 ? dpo::gemm::kTileHalfN : 0);
+                        list[cg - 1].push_back(make_int4(q | flags, b, m0, n0));
+                        k_blocks[cg - 1].push_back(kb);
+                    });
+                }
             }
-            p.tiles = (int)((int64_t)tiles.size() - p.first);
+            p.cg = !list[0].empty() && launch_clocks(k_blocks[0], c->gemm_ctas, 1) <
+                                           launch_clocks(k_blocks[1], c->gemm_pairs, 2)
+                       ? 1
+                       : 2;
+            p.first = (int64_t)tiles.size();
+            p.tiles = (int)list[p.cg - 1].size();
+            tiles.insert(tiles.end(), list[p.cg - 1].begin(), list[p.cg - 1].end());
         }
         c->sets.push_back(ls);
     }
@@ -1090,7 +1150,7 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
         free_ctx(c);
         return mcuda(nullptr, e, "workspace clear");
     }
-    if (e_gemm != cudaSuccess || c->gemm_pairs < 1) {
+    if (e_gemm != cudaSuccess || c->gemm_pairs < 1 || c->gemm_ctas < 1) {
         free_ctx(c);
         return e_gemm != cudaSuccess ? mcuda(nullptr, e_gemm, "GEMM launch configuration")
                                      : mfail(nullptr, DPO_ECUDA, "GEMM kernel cannot be resident");
@@ -1134,13 +1194,11 @@ int launch_gemm(dpo_muon_ctx *c, const LaunchSet &ls, int prod, const GemmJob *j
     L.tiles = c->d_tiles + pr.first;
     L.n_groups = ls.n;
     L.n_tiles = pr.tiles;
-    const bool b_mn = prod == 2;
-    // one CTA pair per co-resident cluster slot (the tile walk assumes every
-    // pair runs at once)
-    const int grid = 2 * std::min(pr.tiles, std::max(1, c->gemm_pairs));
-    const cudaError_t e =
-        dpo::launch_pdl(b_mn ? dpo::gemm::ns_gemm_kernel<true> : dpo::gemm::ns_gemm_kernel<false>,
-                        dim3(grid), dpo::gemm::kThreads, dpo::gemm::kSmemBytes, s, L);
+    // one CTA pair per co-resident cluster slot, or one CTA per SM (the tile
+    // walk assumes that all of them run at once)
+    const int grid = pr.cg * std::min(pr.tiles, pr.cg == 2 ? c->gemm_pairs : c->gemm_ctas);
+    const cudaError_t e = dpo::launch_pdl(gemm_kernel(prod == 2, pr.cg), dim3(grid),
+                                          dpo::gemm::kThreads, dpo::gemm::kSmemBytes, s, L);
     if (c->timing)
         ++c->gemm_launches;
     return e == cudaSuccess ? DPO_OK : mcuda(c, e, "Newton-Schulz GEMM launch");

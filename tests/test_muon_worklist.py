@@ -72,3 +72,21 @@ def test_tiles_half_in_the_padding(cuda_device, steps):
                 assert np.mean(g != r) <= NS_BARS[steps][1], shape
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("shape,copies", [((128, 128), 1), ((129, 257), 1), ((256, 768), 2),
+                                          ((640, 300), 3), ((512, 2048), 40), ((768, 768), 60)])
+def test_tiles_by_single_ctas_and_by_pairs(cuda_device, shape, copies):
+    """One shape from one tile to several rounds of them: the small sets' GEMMs
+    go to single CTAs (128 x 128 tiles), the large sets' to CTA pairs. Two
+    Newton-Schulz steps, so each product reads what the other forms wrote; the
+    first, a middle and the last matrix at the bars of two steps."""
+    p = Pair([shape] * copies, cuda_device, ns_steps=2)
+    try:
+        p.step()
+        got, ref = p.o_pairs()
+        for i in {0, copies // 2, copies - 1}:
+            assert np.linalg.norm(got[i] - ref[i]) <= NS_BARS[2][0] * np.linalg.norm(ref[i]), i
+            assert np.mean(got[i] != ref[i]) <= NS_BARS[2][1], i
+    finally:
+        p.close()
