@@ -87,17 +87,25 @@ template <> struct StashT<kStashBF16> { using T = __nv_bfloat16; };
 
 // ------------------------------------------------------------- cursor ----
 
-// Last tensor whose first packet is <= p (pkt_begin sorted, pkt_begin[0] = 0,
-// pkt_begin[n] = total): for p < total, the tensor holding packet p.
-__device__ __forceinline__ int find_tensor(const int64_t *pkt_begin, int n, int64_t p)
+// Last i with begin[i] <= p in a sorted table (begin[0] <= p), for a p that all
+// 32 lanes of the warp share. Each round the lanes probe 32 evenly spaced
+// entries at once: one load latency up to 32 entries, two up to 1024, where a
+// bisection takes one per halving, before a CTA's first load. GB300, against
+// bisection: a clipped step on 6M elements in 60 tensors 50.0 -> 48.5 us, on 1M
+// in 120 22.2 -> 21.1; five tensors and the large sets are unchanged.
+template <class I>
+__device__ __forceinline__ int warp_find(const I *begin, int n, I p)
 {
-    int lo = 0, hi = n;   // answer in [lo, hi)
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (__ldg(pkt_begin + mid) <= p)
-            lo = mid;
-        else
-            hi = mid;
+    const int lane = threadIdx.x & 31;
+    int lo = 0, len = n;   // answer in [lo, lo + len)
+    while (len > 1) {
+        const int step = (len + 31) / 32;
+        const int i = lane * step;
+        const unsigned below =
+            __ballot_sync(0xFFFFFFFFu, i < len && __ldg(begin + lo + i) <= p);
+        const int k = __popc(below) - 1;   // lane 0's entry is <= p
+        lo += k * step;
+        len = min(step, len - k * step);
     }
     return lo;
 }
@@ -108,9 +116,12 @@ struct Cursor {
     int t;
     int64_t tb, te;   // packet range [tb, te) of tensor t
 
-    __device__ __forceinline__ void seek(const int64_t *pkt_begin, int n, int64_t p)
+    // Every lane of the warp calls this, with growing packets p by lane: the
+    // cursor is left on the tensor of lane 0's packet, and advance() takes it
+    // on to the lane's own.
+    __device__ __forceinline__ void seek(const int64_t *pkt_begin, int n, int64_t p, int64_t total)
     {
-        t = find_tensor(pkt_begin, n, p);
+        t = warp_find(pkt_begin, n, min(__shfl_sync(0xFFFFFFFFu, p, 0), total - 1));
         tb = __ldg(pkt_begin + t);
         te = __ldg(pkt_begin + t + 1);
     }

@@ -62,11 +62,11 @@ __global__ void __launch_bounds__(kNormThreads) grad_sqnorm_kernel(const NormArg
     const int64_t round = (int64_t)gridDim.x * kNormThreads * U;
     const int64_t first = (int64_t)blockIdx.x * kNormThreads * U + threadIdx.x;
     float sum = 0.0f, comp = 0.0f;
-    Cursor c;
+    Cursor c;   // the tables are constant: found before the wait
     const GT *grad = nullptr;
     int64_t numel = 0;
-    if (first < a.total_pkts) {   // the tables are constant: found before the wait
-        c.seek(a.pkt_begin, a.n_tensors, first);
+    if (first - (threadIdx.x & 31) < a.total_pkts) {
+        c.seek(a.pkt_begin, a.n_tensors, first, a.total_pkts);
         grad = static_cast<const GT *>(a.table[c.t].grad);
         numel = a.table[c.t].numel;
     }
@@ -148,10 +148,10 @@ __global__ void __launch_bounds__(kStepThreads) stash_kernel(const StashArgs a)
     using ST = typename StashT<SK>::T;
     const int64_t stride = (int64_t)gridDim.x * kStepThreads;
     int64_t p = (int64_t)blockIdx.x * kStepThreads + threadIdx.x;
+    Cursor c;
+    c.seek(a.pkt_begin, a.n_tensors, p, a.total_pkts);
     if (p >= a.total_pkts)
         return;
-    Cursor c;
-    c.seek(a.pkt_begin, a.n_tensors, p);
     DevTensor d = a.table[c.t];
     for (; p < a.total_pkts; p += stride) {
         if (c.advance(a.pkt_begin, p))

@@ -77,18 +77,6 @@ struct Chunks {
     int elems;                // elements per chunk, a multiple of kRound
 };
 
-// The last matrix i with begin[i] <= c, by every warp at once: the lanes'
-// loads are independent, so the search costs one load latency per 32 matrices
-// (a binary search: one per bisection).
-__device__ __forceinline__ int find_mat(const int *begin, int n, int c)
-{
-    const int lane = threadIdx.x & 31;
-    int cnt = 0;
-    for (int i = 0; i < n; i += 32)
-        cnt += __popc(__ballot_sync(0xFFFFFFFFu, i + lane < n && __ldg(begin + i + lane) <= c));
-    return cnt - 1;
-}
-
 // Row and column of element e of a matrix with `cols` columns. The 64-bit
 // division is a subroutine of some 70 instructions; most matrices fit 32 bits.
 __device__ __forceinline__ void row_col(int64_t e, int64_t cols, bool small, int64_t &i, int64_t &j)
@@ -137,7 +125,7 @@ __global__ void __launch_bounds__(kThreads) muon_momentum_kernel(const MomArgs a
 {
     __shared__ double red[kThreads / 32];
     __shared__ bool last;
-    const int mi = find_mat(a.ch.begin, a.ch.n, (int)blockIdx.x);
+    const int mi = warp_find(a.ch.begin, a.ch.n, (int)blockIdx.x);
     const int c0 = __ldg(a.ch.begin + mi), c1 = __ldg(a.ch.begin + mi + 1);
     const DevMat &d = a.mats[mi];
     pdl_wait();
@@ -243,7 +231,7 @@ __device__ __forceinline__ int tile_at(int i, int j)
 __global__ void __launch_bounds__(kThreads) muon_normalize_kernel(const NormalizeArgs a)
 {
     __shared__ __align__(16) float tile[kTile];
-    const int mi = find_mat(a.tile_begin, a.n, (int)blockIdx.x);
+    const int mi = warp_find(a.tile_begin, a.n, (int)blockIdx.x);
     const DevMat &d = a.mats[mi];
     const int t = (int)blockIdx.x - __ldg(a.tile_begin + mi);
     const bool tall = d.rows > d.cols, packets = d.cols % kPacket == 0;
@@ -379,7 +367,7 @@ template <int SK>
 __global__ void __launch_bounds__(kThreads) muon_apply_kernel(const ApplyArgs a)
 {
     using ST = typename StashT<SK>::T;
-    const int mi = find_mat(a.ch.begin, a.ch.n, (int)blockIdx.x);
+    const int mi = warp_find(a.ch.begin, a.ch.n, (int)blockIdx.x);
     const DevMat &d = a.mats[mi];
     const int64_t n = d.rows * d.cols;
     const int64_t lo = (int64_t)((int)blockIdx.x - __ldg(a.ch.begin + mi)) * a.ch.elems;
@@ -447,7 +435,7 @@ __global__ void __launch_bounds__(kThreads) muon_apply_kernel(const ApplyArgs a)
 // Newton-Schulz output of M' and X_{t+1} the master the real update left.
 __global__ void __launch_bounds__(kThreads) muon_predict_kernel(const ApplyArgs a)
 {
-    const int mi = find_mat(a.ch.begin, a.ch.n, (int)blockIdx.x);
+    const int mi = warp_find(a.ch.begin, a.ch.n, (int)blockIdx.x);
     const DevMat &d = a.mats[mi];
     pdl_wait();
     if (d.sync || d.ef == nullptr)

@@ -145,12 +145,9 @@ __global__ void __launch_bounds__(kStepThreads) fused_step_kernel(const StepArgs
 
     const int64_t stride = (int64_t)gridDim.x * kStepThreads;
     int64_t p = (int64_t)blockIdx.x * kStepThreads + threadIdx.x;
-    Cursor c;
-    DevTensor d{};
-    if (p < a.total_pkts) {   // the tables are constant: found before the wait
-        c.seek(a.pkt_begin, a.n_tensors, p);
-        d = a.table[c.t];
-    }
+    Cursor c;   // the tables are constant: found before the wait
+    c.seek(a.pkt_begin, a.n_tensors, p, a.total_pkts);
+    DevTensor d = a.table[c.t];
     pdl_wait();
     if (p >= a.total_pkts)
         return;
