@@ -120,11 +120,21 @@ def load() -> ctypes.CDLL:
 
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
+
+
+def _current_stream() -> int:
+    """Handle of PyTorch's current stream on the current device. The raw
+    accessor skips the Stream object that torch.cuda.current_stream() makes,
+    2.9 us of the 8.1 us a small step took on the host."""
+    import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
 
 
 def _check(rc: int, ctx) -> None:
