@@ -349,7 +349,7 @@ int dpo_launch_config(const dpo_ctx *ctx, int *step_ctas, int *norm_ctas,
 /*
  * Per-kernel timing, for measurement. With timing on, every dpo_step that
  * launches work records three CUDA events on its stream: before the
- * gradient-norm pass (or the clip-coefficient kernel of a clip source), before
+ * gradient-norm pass (none with a clip source, whose sum the fused step reads), before
  * the fused step, and after it. dpo_get_timing waits for the recorded events,
  * returns the summed milliseconds of the norm interval (*norm_ms, 0 without
  * clipping) and of the fused-step interval (*step_ms) over the *calls timed

@@ -614,15 +614,8 @@ extern "C" int dpo_step(dpo_ctx *c, float lr, void *cuda_stream)
         c->ev_used += 3;
     }
     if (c->total_pkts > 0) {
-        if (c->clip && c->clip_src != nullptr) {
-            const cudaError_t e = dpo::launch_clip_from_sumsq(
-                c->clip_src, (double)c->hp.max_grad_norm, c->d_scalars, s);
-            if (e != cudaSuccess)
-                return cuda_fail(c, e, "clip-coefficient launch");
-        } else if (c->clip) {
-            dpo::NormArgs na{c->d_table, c->d_pkt_begin, c->n, c->total_pkts,
-                             (double)c->hp.max_grad_norm, c->d_partials, c->d_scalars,
-                             nullptr};
+        if (c->clip && c->clip_src == nullptr) {
+            dpo::NormArgs na{c->d_table, c->d_pkt_begin, c->n, c->total_pkts, c->d_partials};
             const cudaError_t e = dpo::launch_norm(c->grad_dt == DPO_BF16, c->norm_grid, na, s);
             if (e != cudaSuccess)
                 return cuda_fail(c, e, "gradient-norm launch");
@@ -669,7 +662,11 @@ extern "C" int dpo_step(dpo_ctx *c, float lr, void *cuda_stream)
         // delayed tensors into the buffer holding x_{t-1}: the stash buffer
         // when t is odd, the param buffer when t is even.
         a.swap = pingpong_on(c) && (t & 1) != 0;
-        a.clip = c->clip ? &c->d_scalars->clip : nullptr;
+        if (c->clip)
+            a.clip = c->clip_src != nullptr
+                         ? dpo::ClipSource{c->clip_src, 1, (double)c->hp.max_grad_norm, c->d_scalars}
+                         : dpo::ClipSource{c->d_partials, c->norm_grid,
+                                           (double)c->hp.max_grad_norm, c->d_scalars};
         if (c->capturable) {   // the per-call scalars come from the device counters
             const dpo::ScalarConsts kc{c->hp.beta1, c->hp.beta2, c->hp.beta3, c->hp.weight_decay,
                                        c->hp.momentum_decay, c->hp.ef_lambda,
@@ -767,10 +764,11 @@ extern "C" int dpo_grad_sqnorm(dpo_ctx *c, double *d_sumsq, void *cuda_stream)
         return fail(c, DPO_EINVAL, "d_sumsq must be an 8-byte aligned device pointer");
     if (c->total_pkts == 0)
         return DPO_OK;
-    dpo::NormArgs na{c->d_table, c->d_pkt_begin, c->n, c->total_pkts, 0.0, c->d_partials,
-                     c->d_scalars, d_sumsq};
-    const cudaError_t e = dpo::launch_norm(c->grad_dt == DPO_BF16, c->norm_grid, na,
-                                           static_cast<cudaStream_t>(cuda_stream));
+    cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+    dpo::NormArgs na{c->d_table, c->d_pkt_begin, c->n, c->total_pkts, c->d_partials};
+    cudaError_t e = dpo::launch_norm(c->grad_dt == DPO_BF16, c->norm_grid, na, s);
+    if (e == cudaSuccess)
+        e = dpo::launch_norm_finish(c->d_partials, c->norm_grid, 0.0, d_sumsq, c->d_scalars, s);
     if (e != cudaSuccess)
         return cuda_fail(c, e, "gradient-norm launch");
     return DPO_OK;

@@ -85,6 +85,26 @@ template <> struct Elem<true> { using T = __nv_bfloat16; };
 template <int SK> struct StashT { using T = float; };
 template <> struct StashT<kStashBF16> { using T = __nv_bfloat16; };
 
+// --------------------------------------------------------------- clip ----
+
+// Norm and clip coefficient min(1, max_norm / (norm + 1e-6)) from a sum of
+// squares; a NaN norm stays NaN and reaches every element.
+__device__ __forceinline__ float clip_coefficient(double total, double max_norm, double &norm)
+{
+    norm = sqrt(total);
+    const double coef = max_norm / (norm + 1e-6);
+    return (float)(coef > 1.0 ? 1.0 : coef);
+}
+
+__device__ __forceinline__ void finish_clip(double total, double max_norm, NormScalars *out)
+{
+    double norm;
+    out->clip = clip_coefficient(total, max_norm, norm);
+    out->norm = norm;
+    if (!isfinite(total))
+        out->flags |= 1u;
+}
+
 // ------------------------------------------------------------- cursor ----
 
 // Last i with begin[i] <= p in a sorted table (begin[0] <= p), for a p that all

@@ -78,6 +78,23 @@ struct ScalarConsts {
     int pingpong;       // ping-pong stash in delayed training
 };
 
+// Device scalars written by the norm pass (one per context).
+struct NormScalars {
+    double norm;          // global gradient norm of the last clipped step
+    float clip;           // clip coefficient used by that step
+    unsigned int flags;   // DPO_FLAG_* bits, sticky until dpo_get_flags reads them
+};
+
+// Where a clipped step takes ||g||^2 from: the norm pass's partial sums, or one
+// sum of its caller's. Every CTA of the step adds them up itself, in the same
+// fixed order, and the first one writes *out.
+struct ClipSource {
+    const double *sums;         // device, or nullptr: no clipping
+    int n;
+    double max_norm;            // clip threshold (> 0)
+    NormScalars *out;
+};
+
 // Scalars of one fused step, precomputed on the host in double and rounded
 // once to fp32 (the per-call ones come from `dev` instead when it is set).
 struct StepArgs {
@@ -107,17 +124,8 @@ struct StepArgs {
     float dc_lambda;            // DC-ASGD strength (0: off)
     int swap;                   // ping-pong stash: write delayed tensors' weights into
                                 // their stash buffer (else their param buffer)
-    const float *clip;          // device clip coefficient, or nullptr
+    ClipSource clip;
     const StepScalars *dev;     // capturable context: the per-call scalars, or nullptr
-};
-
-// Device scalars written by the norm pass (one per context).
-struct NormScalars {
-    double norm;          // global gradient norm of the last clipped step
-    float clip;           // clip coefficient used by that step
-    unsigned int ticket;  // CTA arrival counter, 0 between launches
-    unsigned int flags;   // DPO_FLAG_* bits, sticky until dpo_get_flags reads them
-    unsigned int pad_;
 };
 
 struct NormArgs {
@@ -125,10 +133,7 @@ struct NormArgs {
     const int64_t *pkt_begin;
     int n_tensors;
     int64_t total_pkts;
-    double max_norm;            // clip threshold (> 0)
-    double *partials;           // one per CTA (scratch)
-    NormScalars *out;           // norm, clip coefficient, ticket, flags
-    double *accum;              // non-null: add ||g||^2 to *accum, form no coefficient
+    double *partials;           // one per CTA
 };
 
 struct StashArgs {
@@ -187,11 +192,16 @@ cudaError_t launch_step(Optimizer opt, bool param_bf16, StashKind stash, bool gr
                         Correction corr, bool dc, bool pp, int grid, const StepArgs &a,
                         cudaStream_t s);
 cudaError_t launch_norm(bool grad_bf16, int grid, const NormArgs &a, cudaStream_t s);
+// Adds the n partial sums up (one CTA): into *accum when it is given (one share
+// of a norm over several contexts), else to the norm and clip coefficient of *out.
+cudaError_t launch_norm_finish(const double *partials, int n, double max_norm, double *accum,
+                               NormScalars *out, cudaStream_t s);
 // The per-call scalars of the next step from the device counters, which it
 // advances (one thread; lr from *lr_src when set, else lr).
 cudaError_t launch_step_scalars(StepCounters *cnt, const float *lr_src, float lr,
                                 const ScalarConsts &k, StepScalars *out, cudaStream_t s);
-// Clip coefficient and norm from an external sum of squares (one thread).
+// Clip coefficient and norm from an external sum of squares (one thread; the
+// Muon path's momentum pass reads the coefficient).
 cudaError_t launch_clip_from_sumsq(const double *sumsq, double max_norm, NormScalars *out,
                                    cudaStream_t s);
 cudaError_t launch_stash(bool param_bf16, StashKind stash, int grid, const StashArgs &a,

@@ -1308,6 +1308,23 @@ int orthogonalize(dpo_muon_ctx *c, cudaStream_t s, bool predict)
 
 }  // namespace
 
+namespace {
+
+// ||G||^2 over all matrices: into *accum when it is given, else to the norm and
+// clip coefficient of the context.
+cudaError_t launch_grad_norm(dpo_muon_ctx *c, double *accum, cudaStream_t s)
+{
+    const dpo::NormArgs na{c->d_norm_table, c->d_pkt_begin, c->n, c->total_pkts,
+                           c->d_norm_partials};
+    const cudaError_t e = dpo::launch_norm(c->grad_dt == DPO_BF16, c->norm_grid, na, s);
+    if (e != cudaSuccess)
+        return e;
+    return dpo::launch_norm_finish(c->d_norm_partials, c->norm_grid, c->hp.max_grad_norm, accum,
+                                   c->d_norm_scalars, s);
+}
+
+}  // namespace
+
 extern "C" int dpo_muon_step(dpo_muon_ctx *c, float lr, void *stream)
 {
     if (c == nullptr)
@@ -1332,15 +1349,7 @@ extern "C" int dpo_muon_step(dpo_muon_ctx *c, float lr, void *stream)
         if (e != cudaSuccess)
             return mcuda(c, e, "clip-coefficient launch");
     } else if (clip) {
-        dpo::NormArgs na{};
-        na.table = c->d_norm_table;
-        na.pkt_begin = c->d_pkt_begin;
-        na.n_tensors = c->n;
-        na.total_pkts = c->total_pkts;
-        na.partials = c->d_norm_partials;
-        na.out = c->d_norm_scalars;
-        na.max_norm = c->hp.max_grad_norm;
-        const cudaError_t e = dpo::launch_norm(c->grad_dt == DPO_BF16, c->norm_grid, na, s);
+        const cudaError_t e = launch_grad_norm(c, nullptr, s);
         if (e != cudaSuccess)
             return mcuda(c, e, "norm launch");
     }
@@ -1532,16 +1541,7 @@ extern "C" int dpo_muon_grad_sqnorm(dpo_muon_ctx *c, double *d_sumsq, void *stre
         return mfail(c, DPO_EINVAL, "d_sumsq must be an 8-byte aligned device pointer");
     if (c->total_pkts == 0)
         return DPO_OK;
-    dpo::NormArgs na{};
-    na.table = c->d_norm_table;
-    na.pkt_begin = c->d_pkt_begin;
-    na.n_tensors = c->n;
-    na.total_pkts = c->total_pkts;
-    na.partials = c->d_norm_partials;
-    na.out = c->d_norm_scalars;
-    na.accum = d_sumsq;
-    const cudaError_t e = dpo::launch_norm(c->grad_dt == DPO_BF16, c->norm_grid, na,
-                                           static_cast<cudaStream_t>(stream));
+    const cudaError_t e = launch_grad_norm(c, d_sumsq, static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess)
         return mcuda(c, e, "norm launch");
     return DPO_OK;

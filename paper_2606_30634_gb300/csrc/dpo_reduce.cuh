@@ -105,5 +105,16 @@ __device__ __forceinline__ double block_sum(double x, double *red)
     return r;
 }
 
+// Sum of n partial sums in a fixed order (strided over the NT threads, then the
+// block's tree); valid in thread 0.
+template <int NT>
+__device__ __forceinline__ double ordered_sum(const double *partials, int n, double *red)
+{
+    double acc = 0.0;
+    for (int i = threadIdx.x; i < n; i += NT)
+        acc += __ldcg(partials + i);
+    return block_sum<NT>(acc, red);
+}
+
 }  // namespace
 }  // namespace dpo

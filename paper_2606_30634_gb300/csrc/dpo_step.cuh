@@ -11,7 +11,7 @@
 // stash and no correction.
 #pragma once
 
-#include "dpo_device.cuh"
+#include "dpo_reduce.cuh"
 
 namespace dpo {
 namespace {
@@ -125,6 +125,23 @@ __device__ __forceinline__ float dc_compensate(float lambda, float g, float x, f
     return fmaf(lambda * g * g, x - x_stale, g);
 }
 
+// The clip coefficient of a step, by every CTA from the same sums in the same
+// order; the first CTA leaves the norm's diagnostics.
+__device__ __forceinline__ float step_clip(const ClipSource &c)
+{
+    __shared__ double red[kStepThreads / 32];
+    __shared__ float coef;
+    const double total = ordered_sum<kStepThreads>(c.sums, c.n, red);
+    if (threadIdx.x == 0) {
+        double norm;
+        coef = clip_coefficient(total, c.max_norm, norm);
+        if (blockIdx.x == 0)
+            finish_clip(total, c.max_norm, c.out);
+    }
+    __syncthreads();
+    return coef;
+}
+
 // CORR is a Correction: kCorrNone (standard rule, no history buffer),
 // kCorrEF (lambda-scaled EF; the buffer is read only when lambda != 0),
 // kCorrSapipeSame / kCorrSapipeUpdated (the stash receives the prediction
@@ -149,6 +166,7 @@ __global__ void __launch_bounds__(kStepThreads) fused_step_kernel(const StepArgs
     c.seek(a.pkt_begin, a.n_tensors, p, a.total_pkts);
     DevTensor d = a.table[c.t];
     pdl_wait();
+    const float clip = a.clip.sums != nullptr ? step_clip(a.clip) : 1.0f;
     if (p >= a.total_pkts)
         return;
 
@@ -164,7 +182,6 @@ __global__ void __launch_bounds__(kStepThreads) fused_step_kernel(const StepArgs
                     sc.step_size_next, sc.inv_sqrt_bc2_next, sc.lr, sc.nadam_cg, sc.nadam_cm,
                     a.beta3, a.omb3, sc.inv_sqrt_bc3, sc.adan_c2, sc.nadam_cg_next,
                     sc.nadam_cm_next, sc.inv_sqrt_bc3_next, sc.adan_c2_next, sc.first != 0};
-    const float clip = a.clip != nullptr ? __ldg(a.clip) : 1.0f;
     const bool use_prev = kSapipe || (CORR == kCorrEF && sc.lam != 0.0f);
     const bool ef_now = CORR == kCorrEF && sc.lam != 0.0f;
     const float dc = a.dc_lambda;
