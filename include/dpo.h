@@ -387,9 +387,8 @@ int dpo_get_timing(dpo_ctx *ctx, double *norm_ms, double *step_ms, int64_t *call
  * DPO_NOALLOC_CHUNK_ELEMS elements (smaller chunks for smaller buffers, so
  * they still spread over the SMs); every GPU that loads the library holds
  * it until the process exits. Larger inputs are rejected with DPO_EINVAL.
- * The call allocates nothing: it enqueues one small memset (clearing the
- * scratch's counter, which must start at zero) and one kernel on
- * cuda_stream. The first call on each device looks up the scratch array's
+ * The call allocates nothing: it enqueues one kernel on cuda_stream, or
+ * two for a buffer of more than one chunk. The first call on each device looks up the scratch array's
  * device address (cudaGetSymbolAddress) with that device current and keeps
  * it until the process exits, which assumes the device's primary context
  * lives that long (no cudaDeviceReset in between); make that first call
