@@ -46,6 +46,7 @@ struct dpo_ctx {
     std::vector<dpo_tensor> table;
     int sms = 0;
     int step_grid = 0, norm_grid = 0, stash_grid = 0;
+    int norm_per_thread = 1;   // packets a thread of the norm pass takes per round
     // one device allocation: table | pkt_begin | partials | scalars
     void *dev_block = nullptr;
     DevTensor *d_table = nullptr;
@@ -251,7 +252,20 @@ int set_step_grid(dpo_ctx *c)
         want = 5;
     else
         want = mostly_hist ? 3 : 4;
-    c->step_grid = grid_of(c, std::min(per_sm, want), dpo::kStepThreads);
+    // A set of at most ten CTAs' packets per SM gets one packet per thread: in
+    // two or three rounds the last is nearly empty, and a thread passes over
+    // many small tensors from one round to the next. GB300: a flat 2^20 fp32
+    // step 6.05 -> 5.55 us, a clipped one on 1M elements in 120 tensors 19.7 ->
+    // 15.9; at 20 CTAs' packets NAdam on 3M in 150 tensors loses (30.8 ->
+    // 32.6). A clipped step on few tensors keeps to one wave of CTAs, since
+    // each of them adds the norm's partial sums up first (1M in 2 tensors: 11.2
+    // -> 12.7 with a second wave).
+    const int64_t sms = std::max(1, c->sms), width = dpo::kStepThreads;
+    const bool one_wave = c->total_pkts <= sms * std::max(1, per_sm) * width;
+    if (c->total_pkts <= 10 * sms * width && (one_wave || !c->clip || c->n >= 32))
+        c->step_grid = (int)std::max<int64_t>(1, (c->total_pkts + width - 1) / width);
+    else
+        c->step_grid = grid_of(c, std::min(per_sm, want), dpo::kStepThreads);
     return DPO_OK;
 }
 
@@ -458,7 +472,8 @@ extern "C" int dpo_init(dpo_ctx **out, const dpo_tensor *table, int n_tensors,
         delete c;
         return DPO_ECUDA;
     }
-    c->norm_grid = grid_of(c, per_sm_norm, (int64_t)dpo::kNormThreads * dpo::kNormUnroll);
+    c->norm_per_thread = dpo::norm_per_thread(grad_dtype == DPO_BF16, total_pkts);
+    c->norm_grid = grid_of(c, per_sm_norm, (int64_t)dpo::kNormThreads * c->norm_per_thread);
     c->stash_grid = c->step_grid;
 
     // Device block: table, packet prefix, norm scratch.
@@ -615,7 +630,8 @@ extern "C" int dpo_step(dpo_ctx *c, float lr, void *cuda_stream)
     }
     if (c->total_pkts > 0) {
         if (c->clip && c->clip_src == nullptr) {
-            dpo::NormArgs na{c->d_table, c->d_pkt_begin, c->n, c->total_pkts, c->d_partials};
+            dpo::NormArgs na{c->d_table, c->d_pkt_begin, c->n, c->total_pkts, c->norm_per_thread,
+                             c->d_partials};
             const cudaError_t e = dpo::launch_norm(c->grad_dt == DPO_BF16, c->norm_grid, na, s);
             if (e != cudaSuccess)
                 return cuda_fail(c, e, "gradient-norm launch");
@@ -765,7 +781,8 @@ extern "C" int dpo_grad_sqnorm(dpo_ctx *c, double *d_sumsq, void *cuda_stream)
     if (c->total_pkts == 0)
         return DPO_OK;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    dpo::NormArgs na{c->d_table, c->d_pkt_begin, c->n, c->total_pkts, c->d_partials};
+    dpo::NormArgs na{c->d_table, c->d_pkt_begin, c->n, c->total_pkts, c->norm_per_thread,
+                     c->d_partials};
     cudaError_t e = dpo::launch_norm(c->grad_dt == DPO_BF16, c->norm_grid, na, s);
     if (e == cudaSuccess)
         e = dpo::launch_norm_finish(c->d_partials, c->norm_grid, 0.0, d_sumsq, c->d_scalars, s);

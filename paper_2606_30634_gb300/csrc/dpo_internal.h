@@ -133,6 +133,7 @@ struct NormArgs {
     const int64_t *pkt_begin;
     int n_tensors;
     int64_t total_pkts;
+    int per_thread;             // packets a thread takes per round, 1 .. NormUnroll
     double *partials;           // one per CTA
 };
 
@@ -206,6 +207,11 @@ cudaError_t launch_clip_from_sumsq(const double *sumsq, double max_norm, NormSca
                                    cudaStream_t s);
 cudaError_t launch_stash(bool param_bf16, StashKind stash, int grid, const StashArgs &a,
                          cudaStream_t s);
+
+// Packets per thread and round of the norm pass: the fewest that leave the
+// fused step one partial sum per thread to add up, or as many as a thread can
+// keep in flight.
+int norm_per_thread(bool grad_bf16, int64_t total_pkts);
 
 // Resident CTAs per SM of each kernel at its block size (occupancy query).
 cudaError_t step_ctas_per_sm(Optimizer opt, bool param_bf16, StashKind stash, bool grad_bf16,

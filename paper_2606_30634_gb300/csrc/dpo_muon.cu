@@ -686,6 +686,7 @@ struct dpo_muon_ctx {
     const double *clip_src = nullptr;   // external sum of squares (dpo_muon_set_clip_source)
     int64_t total_pkts = 0;
     int norm_grid = 0;
+    int norm_per_thread = 1;   // packets a thread of the norm pass takes per round
     // GEMM timing (dpo_muon_set_timing): event pairs recorded since the last read
     bool timing = false;
     std::vector<cudaEvent_t> ev_pool;
@@ -979,9 +980,10 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
     c->total_pkts = total_pkts;
     int per_sm_norm = 0;
     dpo::norm_ctas_per_sm(grad_dtype == DPO_BF16, &per_sm_norm);
+    c->norm_per_thread = dpo::norm_per_thread(grad_dtype == DPO_BF16, total_pkts);
     const int64_t norm_groups =
-        (total_pkts + (int64_t)dpo::kNormThreads * dpo::kNormUnroll - 1) /
-        ((int64_t)dpo::kNormThreads * dpo::kNormUnroll);
+        (total_pkts + (int64_t)dpo::kNormThreads * c->norm_per_thread - 1) /
+        ((int64_t)dpo::kNormThreads * c->norm_per_thread);
     c->norm_grid = (int)std::max<int64_t>(
         1, std::min<int64_t>(norm_groups, (int64_t)std::max(1, c->sms) * std::max(1, per_sm_norm)));
 
@@ -1331,7 +1333,7 @@ namespace {
 cudaError_t launch_grad_norm(dpo_muon_ctx *c, double *accum, cudaStream_t s)
 {
     const dpo::NormArgs na{c->d_norm_table, c->d_pkt_begin, c->n, c->total_pkts,
-                           c->d_norm_partials};
+                           c->norm_per_thread, c->d_norm_partials};
     const cudaError_t e = dpo::launch_norm(c->grad_dt == DPO_BF16, c->norm_grid, na, s);
     if (e != cudaSuccess)
         return e;
