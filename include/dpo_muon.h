@@ -42,8 +42,8 @@
  * alive and in place until dpo_muon_destroy. The library allocates, in
  * dpo_muon_init, the Newton-Schulz workspace (bf16, for every matrix: two
  * copies of the iterate, its transpose and two Gram-sized matrices, each
- * dimension padded to a multiple of 256) plus a small table; no other call
- * allocates or synchronizes the host. All launches go to the stream passed in.
+ * dimension padded to a multiple of 256) plus a small table and 16 bytes per
+ * GEMM tile; no other call allocates or synchronizes the host. All launches go to the stream passed in.
  *
  * Errors. Every call returns DPO_OK (0) or a negative DPO_E* code from
  * dpo.h. dpo_muon_last_error gives the message of the last failing call on a
@@ -111,7 +111,7 @@ int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n, dpo_dtype s
  * One iteration with learning rate lr (> 0) for every matrix, enqueued on
  * stream: the norm pass when clipping, the momentum pass, the
  * normalisation pass, 3 ns_steps GEMM launches per matrix shape (or, when
- * some shape's launches are short, per set of up to four shapes sharing each
+ * some shape's launches are short, per set of up to eight shapes sharing each
  * launch) and the update pass. Returns DPO_OK, DPO_EINVAL or DPO_ECUDA.
  */
 int dpo_muon_step(dpo_muon_ctx *ctx, float lr, void *cuda_stream);

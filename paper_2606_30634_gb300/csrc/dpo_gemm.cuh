@@ -15,8 +15,8 @@
 // cluster; CG = 1), where "both CTAs" below is the one. In each CTA:
 //   warp 0      TMA producer: this CTA's 128 x 128 half of the A block and
 //               128 x 128 half of the B block (bf16, 128-byte swizzle, two
-//               64-wide boxes each) into a 3-stage ring, completing on the
-//               leader CTA's mbarrier;
+//               boxes each) into a 3-stage ring, completing on the leader
+//               CTA's mbarrier;
 //   warp 1      allocates 512 TMEM columns (two accumulators) together with
 //               the peer; in the leader, one lane issues
 //               tcgen05.mma.cta_group::2.kind::f16 (M 256, N 256, K 16) eight
@@ -53,7 +53,9 @@ namespace gemm {
 // per stage, and its TMEM holds its BM rows of the accumulator. A stage
 // spans BK = 128 of K as two TMA boxes of kBoxK = 64 (the 128-byte swizzle
 // span); eight MMAs per stage halve the barrier hand-offs per MMA against
-// 64-wide stages, which measured 10% faster on GB300 at equal ring size.
+// 64-wide stages, which are slower on GB300 at equal ring size (six of them:
+// a 7B layer's step 10.1 -> 10.7 ms, four 1B layers 6.5 -> 6.8), and so is a
+// barrier for each half of a stage (6.44 -> 6.51).
 // kTile(2) is that tile. kTile(1) is the tile of a single CTA (128 x 128, the
 // 1-SM MMA, the same stages), for launches of few tiles.
 __host__ __device__ constexpr int kTile(int cg) { return 128 * cg; }
@@ -436,10 +438,11 @@ __device__ __forceinline__ int4 load_tile(const int4 *p)
     return q;
 }
 
-// Persistent: the CTA pairs (clusters of 2) take tiles c, c + pairs, ...
+// Persistent: the CTA pairs (clusters of 2; with CG = 1, the CTAs) take tiles
+// c, c + pairs, ...
 // Within a pair, rank 0 (the leader) issues the MMAs; both ranks load their
 // halves of A and B and drain their own accumulator rows. Two accumulators
-// in TMEM (columns 0-255 and 256-511) let the MMA fill one while the
+// in TMEM, a tile's width of columns each, let the MMA fill one while the
 // epilogues drain the other.
 //   full[s]      (leader) both ranks' TMA bytes of stage s have landed
 //   empty[s]     (each)   the leader's MMAs have finished reading stage s

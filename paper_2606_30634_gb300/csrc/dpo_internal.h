@@ -19,15 +19,15 @@ constexpr uint32_t kFlagWd = 1u;    // DPO_WD_ON
 constexpr uint32_t kFlagSync = 2u;  // DPO_SYNC
 constexpr int kAlign = 32;      // buffer alignment: fp32 packets move as 256-bit accesses
 
-// Fused step and stash kernels: 128-thread CTAs, 3 or 4 resident per SM
-// (the measured table in set_step_grid, dpo_abi.cpp): enough loads in flight
-// to keep HBM3e busy, not so many that DRAM efficiency drops.
+// Fused step and stash kernels: 128-thread CTAs, 3 or 4 resident per SM for
+// sets that stream (the measured table in set_step_grid, dpo_abi.cpp): enough
+// loads in flight to keep HBM3e busy, not so many that DRAM efficiency drops.
 constexpr int kStepThreads = 128;
 
-// Gradient-norm kernel: one read stream, so each thread keeps up to
-// kNormUnroll packets (bf16; half as many fp32 ones) in flight per round.
+// Gradient-norm kernel: one read stream, so each thread keeps several packets in
+// flight per round (NormUnroll, dpo_reduce.cuh; fewer on small sets,
+// norm_per_thread).
 constexpr int kNormThreads = 256;
-constexpr int kNormUnroll = 8;
 
 // Device copy of one table entry.
 struct DevTensor {
