@@ -86,14 +86,15 @@ constexpr unsigned int kErrWaitFull = 1u, kErrWaitEmpty = 2u, kErrWaitDone = 4u,
                        kErrDrain = 8u;
 
 // D is written through the group's store map d (boxes of 32 x 32, 64-byte
-// swizzle) and, with trans, D^T through dt.
+// swizzle), D^T through dt.
 struct Params {
     const __nv_bfloat16 *c;       // M x N addend, or nullptr
     int64_t ldc, c_bstride;
     float alpha, beta;
     int k_blocks;                 // K / BK
     int sym;                      // D is symmetric (M == N): see ns_gemm_kernel
-    int trans;                    // also write D^T (N x M) through the map dt
+    int trans;                    // tiles of tall matrices (kTileTall) write D^T (N x M)
+                                  // through the map dt: see the epilogue
     int stall;                    // test hook: the MMA lane's first accumulator wait
                                   // targets a phase no arrival completes, so it gives up
     unsigned int *err;
@@ -407,7 +408,7 @@ struct GemmGroup {
 // in the kernel (a search over the groups, four divisions) read the launch's
 // parameters through dependent loads and took every role, the MMA lane among
 // them, some 3,900 cycles per tile: a third of a K = 768 tile's time.
-constexpr int kTileGroup = 0xff, kTileHalfM = 0x100, kTileHalfN = 0x200;
+constexpr int kTileGroup = 0xff, kTileHalfM = 0x100, kTileHalfN = 0x200, kTileTall = 0x400;
 
 struct GemmLaunch {
     GemmGroup g[kMaxGroups];
@@ -638,16 +639,23 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
         const int crs = lane >> 2, cg = lane & 3;   // coalesced load: sub-row, granule
         int lt = 0;
         for (int t = pair; t < n_tiles; t += n_pairs) {
-            const int gi = next.x & kTileGroup, b = next.y, m0 = next.z;
+            const int flags = next.x, gi = flags & kTileGroup, b = next.y, m0 = next.z;
             const int n0 = next.w + half * kEpiCols;
             // this warp's rows or columns are all padding: it only passes the
             // accumulator on
-            const bool idle = CG == 2 && ((next.x & kTileHalfM && !leader) ||
-                                          (next.x & kTileHalfN && half));
+            const bool idle = CG == 2 && ((flags & kTileHalfM && !leader) ||
+                                          (flags & kTileHalfN && half));
             if (t + n_pairs < n_tiles)
                 next = load_tile(tiles + t + n_pairs);
             const GemmGroup &G = L.g[gi];
             const Params p = params[gi];   // in registers: the asm statements below clobber memory
+            // D^T instead of D: half the stores of the last product, GPT-2's
+            // step 1768 -> 1749 us.  Single CTAs run the few-tile launches, whose
+            // time is the epilogue's length and not its bytes; there the test
+            // costs more than the stores (two 256 x 512 matrices 97.2 -> 98.3 us),
+            // and every tile writes both.
+            const bool only_t = CG == 2 && p.trans != 0 && (flags & kTileTall);
+            const bool both = p.trans != 0 && CG == 1;
             const int a = lt & 1;
             const int row0 = m0 + (int)rank * BM + q * 32;
             uint4 cpre[kChunks][4];
@@ -685,7 +693,7 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
                 // Uniform over the warp (its rows share row / T) and the chunk
                 // (its columns share col / T).
                 const bool mirror = p.sym && row0 / T < col0 / T;
-                const bool trans = mirror || p.trans != 0;
+                const bool trans = mirror || only_t || both;
                 // Without transposes the two buffers alternate, and only the
                 // chunk before the last one must have been read; a tile's
                 // first chunk may follow one with a transpose.
@@ -726,15 +734,17 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
                     }
                     // each lane rewrites only the row it has read
                 }
+                if (!only_t) {
 #pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    const uint32_t w0 = pack_bf16(v[g * 8 + 0], v[g * 8 + 1]);
-                    const uint32_t w1 = pack_bf16(v[g * 8 + 2], v[g * 8 + 3]);
-                    const uint32_t w2 = pack_bf16(v[g * 8 + 4], v[g * 8 + 5]);
-                    const uint32_t w3 = pack_bf16(v[g * 8 + 6], v[g * 8 + 7]);
-                    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(rb + swz64(lane, g)),
-                                 "r"(w0), "r"(w1), "r"(w2), "r"(w3)
-                                 : "memory");
+                    for (int g = 0; g < 4; ++g) {
+                        const uint32_t w0 = pack_bf16(v[g * 8 + 0], v[g * 8 + 1]);
+                        const uint32_t w1 = pack_bf16(v[g * 8 + 2], v[g * 8 + 3]);
+                        const uint32_t w2 = pack_bf16(v[g * 8 + 4], v[g * 8 + 5]);
+                        const uint32_t w3 = pack_bf16(v[g * 8 + 6], v[g * 8 + 7]);
+                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
+                                     ::"r"(rb + swz64(lane, g)), "r"(w0), "r"(w1), "r"(w2), "r"(w3)
+                                     : "memory");
+                    }
                 }
                 if (trans) {   // element (row, col0 + j) at row j, column lane of the transpose
 #pragma unroll
@@ -749,7 +759,8 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) {
-                    tma_store_3d(&G.d, rb, col0, row0, b);
+                    if (!only_t)
+                        tma_store_3d(&G.d, rb, col0, row0, b);
                     if (trans)
                         tma_store_3d(mirror ? &G.d : &G.dt, tb, row0, col0, b);
                     asm volatile("cp.async.bulk.commit_group;" ::: "memory");

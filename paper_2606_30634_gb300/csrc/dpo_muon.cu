@@ -14,7 +14,7 @@
 //                           every matrix of that shape (dpo_gemm.cuh):
 //                             A = X X^T;  B = c A A + b A;  X <- B X + a X
 //                           (the third reads X MN-major; at the last step it
-//                           also writes X^T, the output of tall matrices)
+//                           writes X^T, their output, for the tall matrices)
 //   muon_apply_kernel       U = lr (r O + wd X_t) and the delayed or EF
 //                           update, stash, history and bf16 weights
 // With the SAPipe-WP updated-state prediction (App. B.1) the step then runs
@@ -954,6 +954,9 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
                         if (cg == 2)
                             flags = (rows <= m0 + side / 2 ? dpo::gemm::kTileHalfM : 0) |
                                     (cols <= n0 + side / 2 ? dpo::gemm::kTileHalfN : 0);
+                        const dpo_matrix &m = mats[g.mats[(size_t)b]];
+                        if (m.rows > m.cols)
+                            flags |= dpo::gemm::kTileTall;
                         list[cg - 1].push_back(make_int4(q | flags, b, m0, n0));
                         k_blocks[cg - 1].push_back(kb);
                     });
@@ -1297,7 +1300,7 @@ int orthogonalize(dpo_muon_ctx *c, cudaStream_t s, bool predict)
                 p.stall = st_aa;
                 aa[q] = GemmJob{&g.a128, &g.a128, &g.st_b, &g.st_b, p};
                 // X <- B X + a X (X read MN-major in place of X^T), and at the
-                // last step X^T for the tall matrices' output
+                // last step X^T, the output, in place of X for the tall matrices
                 p.sym = 0;
                 p.trans = last && g.has_tall ? 1 : 0;
                 p.c = g.x[cur];
