@@ -650,7 +650,7 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
             const GemmGroup &G = L.g[gi];
             const Params p = params[gi];   // in registers: the asm statements below clobber memory
             // D^T instead of D: half the stores of the last product, GPT-2's
-            // step 1768 -> 1749 us.  Single CTAs run the few-tile launches, whose
+            // step 1769 -> 1748 us.  Single CTAs run the few-tile launches, whose
             // time is the epilogue's length and not its bytes; there the test
             // costs more than the stores (two 256 x 512 matrices 97.2 -> 98.3 us),
             // and every tile writes both.
