@@ -232,14 +232,10 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr)
 // Shared-memory descriptor of an MN-major operand tile: rows of 64 bf16
 // (128 bytes) along N with the 128-byte swizzle, one row per K index, 8-row
 // K groups 1024 bytes apart (stride byte offset), and the second 64-column
-// N chunk 16384 bytes further (leading byte offset: one 128-row TMA box). Two
-// such boxes a stage instead of four of 64 rows: the producer lane takes 80 to
-// 95 cycles to issue each, and a stage of B X + a X needed six with A's. GB300,
-// whole step: four 1024-wide layers 1074 -> 1065 us, GPT-2 1767 -> 1764; four
-// 1B layers and a 7B layer within their runs' 1.5 %.
+// N chunk 8192 bytes further (leading byte offset: one 64-row TMA box).
 __device__ __forceinline__ uint64_t smem_desc_mn(uint32_t addr)
 {
-    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(16384 >> 4) << 16) |
+    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(8192 >> 4) << 16) |
            ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
 }
 
@@ -450,7 +446,7 @@ __device__ __forceinline__ int4 load_tile(const int4 *p)
 //   acc_full[a]  (each)   accumulator a holds a finished tile
 //   acc_empty[a] (leader) all epilogue warps of the pair have read it
 // BMN: the B operand is stored N-contiguous (a row-major K x N matrix) and
-// loaded as two boxes of 64 columns per stage, read MN-major by the MMA.
+// loaded as two 64 x 64 boxes per stage, read MN-major by the MMA.
 template <bool BMN, int CG>
 __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
     ns_gemm_kernel(const __grid_constant__ GemmLaunch L)
@@ -549,10 +545,14 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
                         const uint32_t bh = sb + (uint32_t)(s * kBBytes + h * (kBBytes / 2));
                         if (load_a)
                             tma_load_3d<CG>(ah, tma_a, k0, ma, b, fbar);
-                        if (!BMN)
+                        if (BMN) {   // two 64 x 64 boxes: N columns nb_.. and nb_ + 64..
+                            tma_load_3d<CG>(bh, tma_b, nb_, k0, b, fbar);
+                            if (!half_n)
+                                tma_load_3d<CG>(bh + (uint32_t)(kBBytes / 4), tma_b, nb_ + 64, k0,
+                                                b, fbar);
+                        } else {
                             tma_load_3d<CG>(bh, tma_b, k0, nb_, b, fbar);
-                        else if (h == 0 || !half_n)   // columns nb_ + 64 h.., all of the stage's K
-                            tma_load_3d<CG>(bh, tma_b, nb_ + h * 64, kb * BK, b, fbar);
+                        }
                     }
                 }
             }
@@ -599,9 +599,8 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
                         const uint32_t ah = sa + (uint32_t)(s * kABytes + h * (kABytes / 2));
                         const uint32_t bh = sb + (uint32_t)(s * kBBytes + h * (kBBytes / 2));
                         const uint64_t ad = smem_desc(ah + (uint32_t)(kk * 32));
-                        const uint64_t bd =
-                            BMN ? smem_desc_mn(sb + (uint32_t)(s * kBBytes + k * 16 * 128))
-                                : smem_desc(bh + (uint32_t)(kk * 32));
+                        const uint64_t bd = BMN ? smem_desc_mn(bh + (uint32_t)(kk * 16 * 128))
+                                                : smem_desc(bh + (uint32_t)(kk * 32));
                         mma_bf16<CG>(d, ad, bd, idesc, (kb | k) != 0 ? 1u : 0u);
                     }
                     mma_commit<CG>(empty(s));

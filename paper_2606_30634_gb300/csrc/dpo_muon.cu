@@ -630,7 +630,7 @@ struct Group {
     // all of the old X, so the new one goes to the other buffer.
     __nv_bfloat16 *x[2] = {nullptr, nullptr}, *xt = nullptr, *a = nullptr, *b = nullptr;
     CUtensorMap x128[2], a128, b128;   // 128-row K-major boxes: one CTA's half of a pair tile
-    CUtensorMap x_mn[2];               // boxes of 64 columns, BK rows of X read MN-major (B of B X)
+    CUtensorMap x_mn[2];               // 64 x 64 boxes of X read MN-major (B of B X)
     CUtensorMap st_x[2], st_xt, st_a, st_b;   // 32 x 32 store boxes of X, X^T, A, B
 };
 
@@ -1093,8 +1093,8 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
                         make_map(&g.x128[1], g.x[1], g.R, g.W, nb, dpo::gemm::BM) &&
                         make_map(&g.a128, g.a, g.R, g.R, nb, dpo::gemm::BM) &&
                         make_map(&g.b128, g.b, g.R, g.R, nb, dpo::gemm::BM) &&
-                        make_map(&g.x_mn[0], g.x[0], g.R, g.W, nb, dpo::gemm::BK) &&
-                        make_map(&g.x_mn[1], g.x[1], g.R, g.W, nb, dpo::gemm::BK) &&
+                        make_map(&g.x_mn[0], g.x[0], g.R, g.W, nb, 64) &&
+                        make_map(&g.x_mn[1], g.x[1], g.R, g.W, nb, 64) &&
                         make_store_map(&g.st_x[0], g.x[0], g.R, g.W, nb) &&
                         make_store_map(&g.st_x[1], g.x[1], g.R, g.W, nb) &&
                         make_store_map(&g.st_xt, g.xt, g.W, g.R, nb) &&
