@@ -61,14 +61,14 @@ namespace gemm {
 __host__ __device__ constexpr int kTile(int cg) { return 128 * cg; }
 constexpr int TM = kTile(2), TN = kTile(2);
 constexpr int BM = 128, BH = 128, BK = 128, kBoxK = 64, kStages = 3;
-// Epilogue warps: two per TMEM lane quarter, each taking half of the tile's
-// columns: a tile's epilogue is a serial chain per warp (TMEM read, addend,
-// staging, store), which the 6 k-blocks of a K = 768 tile do not hide at four
-// warps. GB300, four against eight warps, whole step: GPT-2 1816 -> 1777 us,
-// twelve 768-wide layers 1525 -> 1486, two 256x768 matrices 145 -> 133; a 7B
-// layer, whose tiles have 32 k-blocks, is unchanged.
+// Epilogue warps, at most: two per TMEM lane quarter, each taking half of the
+// tile's columns: a tile's epilogue is a serial chain per warp (TMEM read,
+// addend, staging, store), which the 6 k-blocks of a K = 768 tile do not hide at
+// four warps. GB300, four against eight warps, whole step: GPT-2 1816 -> 1777 us,
+// twelve 768-wide layers 1525 -> 1486, two 256x768 matrices 145 -> 133. Long
+// launches with long K run four (kLongBlocks in dpo_muon.cu).
 constexpr int kEpiWarps = 8;
-constexpr int kThreads = 64 + 32 * kEpiWarps;
+__host__ __device__ constexpr int gemm_threads(int ew) { return 64 + 32 * ew; }
 constexpr int kABytes = BM * BK * 2;                 // 32 KiB
 constexpr int kBBytes = BH * BK * 2;                 // 32 KiB
 constexpr int kStageBytes = kABytes + kBBytes;       // 64 KiB per CTA
@@ -445,14 +445,15 @@ __device__ __forceinline__ int4 load_tile(const int4 *p)
 //   empty[s]     (each)   the leader's MMAs have finished reading stage s
 //   acc_full[a]  (each)   accumulator a holds a finished tile
 //   acc_empty[a] (leader) all epilogue warps of the pair have read it
+// EW: epilogue warps, 8 or 4; with 4 each takes both halves of the columns.
 // BMN: the B operand is stored N-contiguous (a row-major K x N matrix) and
 // loaded as two 64 x 64 boxes per stage, read MN-major by the MMA.
-template <bool BMN, int CG>
-__global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
+template <bool BMN, int CG, int EW>
+__global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(gemm_threads(EW), 1)
     ns_gemm_kernel(const __grid_constant__ GemmLaunch L)
 {
     constexpr int T = kTile(CG);                   // tile side, TMEM columns of an accumulator
-    constexpr int kEpiCols = T * 4 / kEpiWarps;    // columns per epilogue warp
+    constexpr int kEpiCols = T / 2;                // columns an epilogue warp drains at a time
     unsigned int *const err = L.g[0].p.err;   // err and stall are the launch's
     const int stall = L.g[0].p.stall;
     extern __shared__ uint8_t smem_raw[];
@@ -481,7 +482,7 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(acc_full(a), 1);
-            mbar_init(acc_empty(a), CG * kEpiWarps);   // one arrival per epilogue warp of the pair
+            mbar_init(acc_empty(a), CG * EW);   // one arrival per epilogue warp of the pair
         }
         aborted = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -619,13 +620,14 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
     } else {
         // Epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 = this CTA's
         // tile rows m0 + BM rank + 32 (w % 4) + lane, and the half of the tile's
-        // columns that (w - 2) / 4 names. Each 32 x 32 chunk is staged in
+        // columns that (w - 2) / 4 names (of four warps: both halves in turn).
+        // Each 32 x 32 chunk is staged in
         // shared memory (and its transpose, for a mirrored or a transposed
         // output) and written by one TMA store per box from lane 0; direct
         // stores from 32 rows at a time cost the MMAs a fifth of their rate
         // on GB300. Lane 0 waits until the buffers it is about to rewrite have
         // been read.
-        const int q = warp & 3, half = (warp - 2) >> 2;
+        const int q = warp & 3, half0 = (warp - 2) >> 2;
         const uint32_t wbuf =
             ring + (uint32_t)(kStages * kStageBytes + (warp - 2) * 2 * kChunkBytes);
         // The addend C (c A A + b A, B X + a X) of all the warp's chunks is
@@ -639,11 +641,7 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
         int lt = 0;
         for (int t = pair; t < n_tiles; t += n_pairs) {
             const int flags = next.x, gi = flags & kTileGroup, b = next.y, m0 = next.z;
-            const int n0 = next.w + half * kEpiCols;
-            // this warp's rows or columns are all padding: it only passes the
-            // accumulator on
-            const bool idle = CG == 2 && ((flags & kTileHalfM && !leader) ||
-                                          (flags & kTileHalfN && half));
+            const int tile_n0 = next.w;
             if (t + n_pairs < n_tiles)
                 next = load_tile(tiles + t + n_pairs);
             const GemmGroup &G = L.g[gi];
@@ -657,114 +655,129 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
             const bool both = p.trans != 0 && CG == 1;
             const int a = lt & 1;
             const int row0 = m0 + (int)rank * BM + q * 32;
-            uint4 cpre[kChunks][4];
-            if (p.c != nullptr && !idle) {
-                // C at (row0 + crs, n0 + 8 cg); rows 8 i further for i = 0..3
-                const __nv_bfloat16 *crow = p.c + (int64_t)b * p.c_bstride +
-                                            (int64_t)(row0 + crs) * p.ldc + n0 + cg * 8;
+            bool seen = true;
 #pragma unroll
-                for (int c = 0; c < kChunks; ++c)
+            for (int h = 0; h < kEpiWarps / EW; ++h) {
+                const int half = half0 + h, n0 = tile_n0 + half * kEpiCols;
+                // these rows or columns are all padding: the warp only passes
+                // the accumulator on
+                const bool idle = CG == 2 && ((flags & kTileHalfM && !leader) ||
+                                              (flags & kTileHalfN && half));
+                uint4 cpre[kChunks][4];
+                if (p.c != nullptr && !idle) {
+                    // C at (row0 + crs, n0 + 8 cg); rows 8 i further for i = 0..3
+                    const __nv_bfloat16 *crow = p.c + (int64_t)b * p.c_bstride +
+                                                (int64_t)(row0 + crs) * p.ldc + n0 + cg * 8;
 #pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        cpre[c][i] = load_c(crow + 8 * i * p.ldc + c * 32);
-            }
-            const bool seen = mbar_wait(acc_full(a), (uint32_t)(lt >> 1) & 1u);
-            if (!seen)
-                atomicOr(err, kErrWaitDone);
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            // tcgen05.ld is warp-collective: the whole warp goes on, or none of it.
-            if (!__all_sync(0xFFFFFFFFu, seen && !*(volatile int *)&aborted))
-                break;
-            const uint32_t acc =
-                tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * T + half * kEpiCols);
-            if (!idle)
+                    for (int c = 0; c < kChunks; ++c)
 #pragma unroll
-            for (int ch = 0; ch < kChunks; ++ch) {
-                uint32_t r[32];
-                tmem_ld32(acc + (uint32_t)(ch * 32), r);
-                float v[32];
-#pragma unroll
-                for (int j = 0; j < 32; ++j)
-                    v[j] = p.alpha * __uint_as_float(r[j]);
-                const int col0 = n0 + ch * 32;
-                // Mirror of a symmetric product: (col, row) lies in the tile
-                // (col / T, row / T), not computed when row / T < col / T.
-                // Uniform over the warp (its rows share row / T) and the chunk
-                // (its columns share col / T).
-                const bool mirror = p.sym && row0 / T < col0 / T;
-                const bool trans = mirror || only_t || both;
-                // Without transposes the two buffers alternate, and only the
-                // chunk before the last one must have been read; a tile's
-                // first chunk may follow one with a transpose.
-                const uint32_t rb = wbuf + (trans ? 0u : (uint32_t)((ch & 1) * kChunkBytes));
-                const uint32_t tb = wbuf + (uint32_t)kChunkBytes;
-                if (lane == 0) {
-                    if (trans || ch == 0)
-                        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-                    else
-                        asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                        for (int i = 0; i < 4; ++i)
+                            cpre[c][i] = load_c(crow + 8 * i * p.ldc + c * 32);
                 }
-                __syncwarp();
-                if (p.c != nullptr) {
-                    // the coalesced chunk of C into rb, then this lane's row out
+                if (h == 0) {
+                    seen = mbar_wait(acc_full(a), (uint32_t)(lt >> 1) & 1u);
+                    if (!seen)
+                        atomicOr(err, kErrWaitDone);
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    // tcgen05.ld is warp-collective: the whole warp goes on, or
+                    // none of it.
+                    seen = __all_sync(0xFFFFFFFFu, seen && !*(volatile int *)&aborted);
+                }
+                if (!seen)
+                    break;
+                const uint32_t acc =
+                    tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * T + half * kEpiCols);
+                if (!idle)
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const uint4 cv = cpre[ch][i];
-                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
-                                     ::"r"(rb + swz64(crs + 8 * i, cg)), "r"(cv.x), "r"(cv.y),
-                                       "r"(cv.z), "r"(cv.w)
-                                     : "memory");
+                for (int ch = 0; ch < kChunks; ++ch) {
+                    uint32_t r[32];
+                    tmem_ld32(acc + (uint32_t)(ch * 32), r);
+                    float v[32];
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        v[j] = p.alpha * __uint_as_float(r[j]);
+                    const int col0 = n0 + ch * 32;
+                    // Mirror of a symmetric product: (col, row) lies in the tile
+                    // (col / T, row / T), not computed when row / T < col / T.
+                    // Uniform over the warp (its rows share row / T) and the chunk
+                    // (its columns share col / T).
+                    const bool mirror = p.sym && row0 / T < col0 / T;
+                    const bool trans = mirror || only_t || both;
+                    // Without transposes the two buffers alternate, and only the
+                    // chunk before the last one must have been read; a tile's
+                    // first chunk may follow one with a transpose.
+                    const uint32_t rb = wbuf + (trans ? 0u : (uint32_t)((ch & 1) * kChunkBytes));
+                    const uint32_t tb = wbuf + (uint32_t)kChunkBytes;
+                    if (lane == 0) {
+                        if (trans || ch == 0)
+                            asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                        else
+                            asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
                     }
                     __syncwarp();
+                    if (p.c != nullptr) {
+                        // the coalesced chunk of C into rb, then this lane's row out
 #pragma unroll
-                    for (int g = 0; g < 4; ++g) {
-                        uint4 cv;
-                        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-                                     : "=r"(cv.x), "=r"(cv.y), "=r"(cv.z), "=r"(cv.w)
-                                     : "r"(rb + swz64(lane, g))
-                                     : "memory");
-                        const __nv_bfloat162 *c2 = reinterpret_cast<const __nv_bfloat162 *>(&cv);
+                        for (int i = 0; i < 4; ++i) {
+                            const uint4 cv = cpre[ch][i];
+                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
+                                         ::"r"(rb + swz64(crs + 8 * i, cg)), "r"(cv.x), "r"(cv.y),
+                                           "r"(cv.z), "r"(cv.w)
+                                         : "memory");
+                        }
+                        __syncwarp();
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float2 f = __bfloat1622float2(c2[e]);
-                            v[g * 8 + 2 * e] = fmaf(p.beta, f.x, v[g * 8 + 2 * e]);
-                            v[g * 8 + 2 * e + 1] = fmaf(p.beta, f.y, v[g * 8 + 2 * e + 1]);
+                        for (int g = 0; g < 4; ++g) {
+                            uint4 cv;
+                            asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                                         : "=r"(cv.x), "=r"(cv.y), "=r"(cv.z), "=r"(cv.w)
+                                         : "r"(rb + swz64(lane, g))
+                                         : "memory");
+                            const __nv_bfloat162 *c2 = reinterpret_cast<const __nv_bfloat162 *>(&cv);
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const float2 f = __bfloat1622float2(c2[e]);
+                                v[g * 8 + 2 * e] = fmaf(p.beta, f.x, v[g * 8 + 2 * e]);
+                                v[g * 8 + 2 * e + 1] = fmaf(p.beta, f.y, v[g * 8 + 2 * e + 1]);
+                            }
+                        }
+                        // each lane rewrites only the row it has read
+                    }
+                    if (!only_t) {
+#pragma unroll
+                        for (int g = 0; g < 4; ++g) {
+                            const uint32_t w0 = pack_bf16(v[g * 8 + 0], v[g * 8 + 1]);
+                            const uint32_t w1 = pack_bf16(v[g * 8 + 2], v[g * 8 + 3]);
+                            const uint32_t w2 = pack_bf16(v[g * 8 + 4], v[g * 8 + 5]);
+                            const uint32_t w3 = pack_bf16(v[g * 8 + 6], v[g * 8 + 7]);
+                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
+                                         ::"r"(rb + swz64(lane, g)), "r"(w0), "r"(w1), "r"(w2), "r"(w3)
+                                         : "memory");
                         }
                     }
-                    // each lane rewrites only the row it has read
-                }
-                if (!only_t) {
+                    if (trans) {   // element (row, col0 + j) at row j, column lane of the transpose
 #pragma unroll
-                    for (int g = 0; g < 4; ++g) {
-                        const uint32_t w0 = pack_bf16(v[g * 8 + 0], v[g * 8 + 1]);
-                        const uint32_t w1 = pack_bf16(v[g * 8 + 2], v[g * 8 + 3]);
-                        const uint32_t w2 = pack_bf16(v[g * 8 + 4], v[g * 8 + 5]);
-                        const uint32_t w3 = pack_bf16(v[g * 8 + 6], v[g * 8 + 7]);
-                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
-                                     ::"r"(rb + swz64(lane, g)), "r"(w0), "r"(w1), "r"(w2), "r"(w3)
-                                     : "memory");
+                        for (int j = 0; j < 32; ++j) {
+                            const __nv_bfloat16 h = __float2bfloat16_rn(v[j]);
+                            asm volatile("st.shared.b16 [%0], %1;" ::"r"(tb + swz64(j, lane >> 3) +
+                                                                          (uint32_t)((lane & 7) * 2)),
+                                         "h"(*reinterpret_cast<const uint16_t *>(&h))
+                                         : "memory");
+                        }
                     }
-                }
-                if (trans) {   // element (row, col0 + j) at row j, column lane of the transpose
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const __nv_bfloat16 h = __float2bfloat16_rn(v[j]);
-                        asm volatile("st.shared.b16 [%0], %1;" ::"r"(tb + swz64(j, lane >> 3) +
-                                                                      (uint32_t)((lane & 7) * 2)),
-                                     "h"(*reinterpret_cast<const uint16_t *>(&h))
-                                     : "memory");
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) {
+                        if (!only_t)
+                            tma_store_3d(&G.d, rb, col0, row0, b);
+                        if (trans)
+                            tma_store_3d(mirror ? &G.d : &G.dt, tb, row0, col0, b);
+                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                     }
-                }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) {
-                    if (!only_t)
-                        tma_store_3d(&G.d, rb, col0, row0, b);
-                    if (trans)
-                        tma_store_3d(mirror ? &G.d : &G.dt, tb, row0, col0, b);
-                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                 }
             }
+            if (!seen)
+                break;
             // this warp's rows of the accumulator are read: release them to
             // the leader's MMA lane
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");

@@ -570,11 +570,15 @@ bool make_store_map(CUtensorMap *m, void *base, int64_t rows, int64_t cols, int6
 
 using GemmFn = void (*)(dpo::gemm::GemmLaunch);
 
-GemmFn gemm_kernel(bool b_mn, int cg)
+// By CTAs per tile and epilogue warps (single CTAs always have eight).
+GemmFn gemm_kernel(bool b_mn, int cg, int ew)
 {
-    if (cg == 2)
-        return b_mn ? dpo::gemm::ns_gemm_kernel<true, 2> : dpo::gemm::ns_gemm_kernel<false, 2>;
-    return b_mn ? dpo::gemm::ns_gemm_kernel<true, 1> : dpo::gemm::ns_gemm_kernel<false, 1>;
+    using dpo::gemm::ns_gemm_kernel;
+    if (cg == 1)
+        return b_mn ? ns_gemm_kernel<true, 1, 8> : ns_gemm_kernel<false, 1, 8>;
+    if (ew == 4)
+        return b_mn ? ns_gemm_kernel<true, 2, 4> : ns_gemm_kernel<false, 2, 4>;
+    return b_mn ? ns_gemm_kernel<true, 2, 8> : ns_gemm_kernel<false, 2, 8>;
 }
 
 // Estimated clocks of a launch over tiles with these K blocks, dealt round-robin
@@ -603,6 +607,14 @@ int64_t launch_clocks(const std::vector<int> &k_blocks, int slots, int cg)
     return worst;
 }
 
+// A pair launch of more than kLongRounds rounds of tiles, each of at least
+// kLongBlocks K blocks, is drained by four epilogue warps instead of eight: the
+// next tile's mainloop hides either, and at the power cap the eight cost clocks.
+// GB300, eight against four warps, whole step: the 7B set 332.0 -> 323.8 ms, a 7B
+// layer 10370 -> 10180 us, six 2048-wide layers 8107 -> 8063 us. Shorter K needs
+// the eight (kEpiWarps), and so does a launch whose last tile is much of it.
+constexpr int kLongBlocks = 16, kLongRounds = 4;
+
 // Rounds of single-CTA tiles above which a launch goes to the pairs unweighed.
 constexpr int64_t kFewRounds = 4;
 
@@ -619,6 +631,7 @@ struct LaunchSet {
         int64_t first = 0;                  // first entry of the tile table
         int tiles = 0;
         int cg = 2;                         // CTAs per tile: 256 x 256 pairs, or 128 x 128
+        int ew = 8;                         // epilogue warps of a CTA
     } prod[3];
 };
 
@@ -884,22 +897,22 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
     // would come).
     c->gemm_pairs = c->gemm_ctas = 1 << 30;
     cudaError_t e_gemm = cudaSuccess;
-    for (int cg = 1; cg <= 2 && e_gemm == cudaSuccess; ++cg)
-        for (int mn = 0; mn < 2 && e_gemm == cudaSuccess; ++mn) {
-            const void *fn = (const void *)gemm_kernel(mn != 0, cg);
-            e_gemm = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          dpo::gemm::kSmemBytes);
-            int n_res = 0;
-            if (e_gemm == cudaSuccess) {
-                cudaLaunchConfig_t cfg = {};
-                cfg.gridDim = dim3(2 * std::max(1, c->sms / 2));
-                cfg.blockDim = dim3(dpo::gemm::kThreads);
-                cfg.dynamicSmemBytes = dpo::gemm::kSmemBytes;
-                e_gemm = cudaOccupancyMaxActiveClusters(&n_res, fn, &cfg);
-            }
-            int &have = cg == 2 ? c->gemm_pairs : c->gemm_ctas;
-            have = std::min(have, n_res);
+    for (int form = 0; form < 6 && e_gemm == cudaSuccess; ++form) {
+        const int cg = form < 2 ? 1 : 2, ew = form < 4 ? 8 : 4;
+        const void *fn = (const void *)gemm_kernel(form & 1, cg, ew);
+        e_gemm = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      dpo::gemm::kSmemBytes);
+        int n_res = 0;
+        if (e_gemm == cudaSuccess) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(2 * std::max(1, c->sms / 2));
+            cfg.blockDim = dim3(dpo::gemm::gemm_threads(ew));
+            cfg.dynamicSmemBytes = dpo::gemm::kSmemBytes;
+            e_gemm = cudaOccupancyMaxActiveClusters(&n_res, fn, &cfg);
         }
+        int &have = cg == 2 ? c->gemm_pairs : c->gemm_ctas;
+        have = std::min(have, n_res);
+    }
     // When some shape group's launches are short (at most 16 rounds of tiles
     // over the CTA pairs), each product of a Newton-Schulz step covers all
     // shape groups in one launch: one group's tiles fill the pairs another
@@ -968,6 +981,9 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
                        : 2;
             p.first = (int64_t)tiles.size();
             p.tiles = (int)list[p.cg - 1].size();
+            if (p.cg == 2 && p.tiles > kLongRounds * c->gemm_pairs &&
+                *std::min_element(k_blocks[1].begin(), k_blocks[1].end()) >= kLongBlocks)
+                p.ew = 4;
             tiles.insert(tiles.end(), list[p.cg - 1].begin(), list[p.cg - 1].end());
         }
         c->sets.push_back(ls);
@@ -1205,8 +1221,9 @@ int launch_gemm(dpo_muon_ctx *c, const LaunchSet &ls, int prod, const GemmJob *j
     // one CTA pair per co-resident cluster slot, or one CTA per SM (the tile
     // walk assumes that all of them run at once)
     const int grid = pr.cg * std::min(pr.tiles, pr.cg == 2 ? c->gemm_pairs : c->gemm_ctas);
-    const cudaError_t e = dpo::launch_pdl(gemm_kernel(prod == 2, pr.cg), dim3(grid),
-                                          dpo::gemm::kThreads, dpo::gemm::kSmemBytes, s, L);
+    const cudaError_t e =
+        dpo::launch_pdl(gemm_kernel(prod == 2, pr.cg, pr.ew), dim3(grid),
+                        dpo::gemm::gemm_threads(pr.ew), dpo::gemm::kSmemBytes, s, L);
     if (c->timing)
         ++c->gemm_launches;
     return e == cudaSuccess ? DPO_OK : mcuda(c, e, "Newton-Schulz GEMM launch");

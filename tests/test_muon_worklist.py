@@ -8,7 +8,9 @@ from __future__ import annotations
 
 import numpy as np
 import pytest
+import torch
 
+from paper_2606_30634_gb300 import muon
 from parity_util import TOL_ONE_STEP, TOL_RUN, rel_err
 from test_muon_parity import F, NS_BARS, Pair, _flat, close_with_flips
 
@@ -90,3 +92,29 @@ def test_tiles_by_single_ctas_and_by_pairs(cuda_device, shape, copies):
             assert np.mean(got[i] != ref[i]) <= NS_BARS[2][1], i
     finally:
         p.close()
+
+
+def test_four_epilogue_warps_match_eight(cuda_device):
+    """K of 4098 and 4100 (33 blocks, the last nearly empty): a wide and a tall
+    matrix together are 578 pair tiles in B X + a X, which four epilogue warps
+    drain; each alone is 289, which eight do. The same tiles either way, so the
+    same bits."""
+    shapes = [(4098, 4100), (4100, 4098)]
+    gen = torch.Generator().manual_seed(7)
+    grads = [torch.randn(s, generator=gen) for s in shapes]
+
+    def outputs(which):
+        m = muon.DelayedMuon([shapes[i] for i in which], ns_steps=2, lr=0.02, momentum=0.95,
+                             device=cuda_device, x0=[torch.zeros(shapes[i]) for i in which])
+        try:
+            for q, i in enumerate(which):
+                m.grads(q).copy_(grads[i])
+            m.step()
+            torch.cuda.synchronize()
+            return [m.last_update(q).clone() for q in range(len(which))]
+        finally:
+            m.close()
+
+    for i, got in enumerate(outputs([0, 1])):
+        assert torch.equal(got, outputs([i])[0]), shapes[i]
+        assert got.float().abs().sum() > 0
