@@ -21,6 +21,11 @@ namespace {
 // kernel's parameters and the tables uploaded at init are read before it. It
 // returns once all earlier work of the stream is complete and visible (the
 // kernel before completed only after its own wait, and so on).
+// So a kernel is live while the one before it still writes, and what that one
+// writes is not read-only for the kernel's lifetime: the non-coherent path
+// (ld_table; ld.global.nc) is for the tables of init alone. Everything else is
+// read by an ordinary load: a plain one, which the wait's memory clobber keeps
+// behind it, or a volatile asm, which keeps its place among volatile asms.
 // No kernel asks for its successor earlier than that
 // (griddepcontrol.launch_dependents at its start): CTAs that arrive while
 // others still run are spread unevenly over the SMs, and the persistent
@@ -29,6 +34,9 @@ namespace {
 // Newton-Schulz step 1679 / 1565; only a clipped step on 74 thousand elements
 // gained (9.5 / 10.0).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Entry of a table uploaded at init, which no kernel writes.
+template <class I> __device__ __forceinline__ I ld_table(const I *p) { return __ldg(p); }
 
 // ---------------------------------------------------------------- I/O ----
 // fp32 packet: one 32-byte (256-bit) load or store per thread.
@@ -50,9 +58,18 @@ __device__ __forceinline__ void st8(float *p, const float (&r)[8])
 }
 
 // bf16 packet: one 16-byte load or store; values widen exactly to fp32.
+__device__ __forceinline__ uint4 ld_packet(const __nv_bfloat16 *p)
+{
+    uint4 q;
+    asm volatile("ld.global.cs.v4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(q.x), "=r"(q.y), "=r"(q.z), "=r"(q.w)
+                 : "l"(p));
+    return q;
+}
+
 __device__ __forceinline__ void ld8(const __nv_bfloat16 *p, float (&r)[8])
 {
-    const uint4 q = __ldcs(reinterpret_cast<const uint4 *>(p));
+    const uint4 q = ld_packet(p);
     const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -74,8 +91,25 @@ __device__ __forceinline__ void st8(__nv_bfloat16 *p, const float (&r)[8])
     __stcs(reinterpret_cast<uint4 *>(p), q);
 }
 
-__device__ __forceinline__ float ld1(const float *p) { return __ldcs(p); }
-__device__ __forceinline__ float ld1(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
+__device__ __forceinline__ float ld1(const float *p)
+{
+    float x;
+    asm volatile("ld.global.cs.f32 %0, [%1];" : "=f"(x) : "l"(p));
+    return x;
+}
+__device__ __forceinline__ float ld1(const __nv_bfloat16 *p)
+{
+    uint16_t x;
+    asm volatile("ld.global.b16 %0, [%1];" : "=h"(x) : "l"(p));
+    return __uint_as_float((uint32_t)x << 16);
+}
+// A partial sum that another CTA wrote, from L2.
+__device__ __forceinline__ double ld_partial(const double *p)
+{
+    double x;
+    asm volatile("ld.global.cg.f64 %0, [%1];" : "=d"(x) : "l"(p) : "memory");
+    return x;
+}
 __device__ __forceinline__ void st1(float *p, float x) { __stcs(p, x); }
 __device__ __forceinline__ void st1(__nv_bfloat16 *p, float x) { *p = __float2bfloat16_rn(x); }
 
@@ -122,7 +156,7 @@ __device__ __forceinline__ int warp_find(const I *begin, int n, I p)
         const int step = (len + 31) / 32;
         const int i = lane * step;
         const unsigned below =
-            __ballot_sync(0xFFFFFFFFu, i < len && __ldg(begin + lo + i) <= p);
+            __ballot_sync(0xFFFFFFFFu, i < len && ld_table(begin + lo + i) <= p);
         const int k = __popc(below) - 1;   // lane 0's entry is <= p
         lo += k * step;
         len = min(step, len - k * step);
@@ -142,8 +176,8 @@ struct Cursor {
     __device__ __forceinline__ void seek(const int64_t *pkt_begin, int n, int64_t p, int64_t total)
     {
         t = warp_find(pkt_begin, n, min(__shfl_sync(0xFFFFFFFFu, p, 0), total - 1));
-        tb = __ldg(pkt_begin + t);
-        te = __ldg(pkt_begin + t + 1);
+        tb = ld_table(pkt_begin + t);
+        te = ld_table(pkt_begin + t + 1);
     }
     // true when the packet moved to another tensor (p < total)
     __device__ __forceinline__ bool advance(const int64_t *pkt_begin, int64_t p)
@@ -153,7 +187,7 @@ struct Cursor {
         do {
             ++t;
             tb = te;
-            te = __ldg(pkt_begin + t + 1);
+            te = ld_table(pkt_begin + t + 1);
         } while (p >= te);
         return true;
     }

@@ -414,18 +414,20 @@ struct GemmLaunch {
 };
 
 // 16 bytes of the addend, pinned where it is written, before the wait for the
-// accumulator.
+// accumulator. Through L1, which keeps the other half of each line for the next
+// chunk's load: with L1::no_allocate GPT-2's step takes 1766 us against 1750, two
+// 256 x 768 matrices 100.9 against 99.9.
 __device__ __forceinline__ uint4 load_c(const __nv_bfloat16 *p)
 {
     uint4 q;
-    asm volatile("ld.global.nc.v4.b32 {%0, %1, %2, %3}, [%4];"
+    asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];"
                  : "=r"(q.x), "=r"(q.y), "=r"(q.z), "=r"(q.w)
                  : "l"(p));
     return q;
 }
 
-// Entry t of the tile table, pinned where it is written (a plain load may be
-// moved down to its first use, a tile later).
+// Entry t of the tile table (made at init), pinned where it is written (a plain
+// load may be moved down to its first use, a tile later).
 __device__ __forceinline__ int4 load_tile(const int4 *p)
 {
     int4 q;

@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(kThreads) muon_momentum_kernel(const MomArgs a
     __shared__ double red[kThreads / 32];
     __shared__ bool last;
     const int mi = warp_find(a.ch.begin, a.ch.n, (int)blockIdx.x);
-    const int c0 = __ldg(a.ch.begin + mi), c1 = __ldg(a.ch.begin + mi + 1);
+    const int c0 = ld_table(a.ch.begin + mi), c1 = ld_table(a.ch.begin + mi + 1);
     const DevMat &d = a.mats[mi];
     pdl_wait();
     // the prediction pass leaves a synchronous matrix (and its history) alone
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(kThreads) muon_momentum_kernel(const MomArgs a
     const int64_t lo = (int64_t)((int)blockIdx.x - c0) * a.ch.elems;
     float sum = 0.0f, comp = 0.0f;
     if (lo < n) {
-        const float clip = a.clip != nullptr ? __ldg(a.clip) : 1.0f;
+        const float clip = a.clip != nullptr ? *a.clip : 1.0f;
         const int64_t hi = lo + a.ch.elems < n ? lo + a.ch.elems : n;
         const GT *grad = static_cast<const GT *>(d.grad);
         for (int64_t e = lo + (int64_t)threadIdx.x * kPacket; e < hi; e += (int64_t)kThreads * kPacket) {
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(kThreads) muon_momentum_kernel(const MomArgs a
     __threadfence();
     double acc = 0.0;
     for (int c = c0 + (int)threadIdx.x; c < c1; c += kThreads)
-        acc += __ldcg(a.partials + c);
+        acc += ld_partial(a.partials + c);
     const double total = block_sum<kThreads>(acc, red);
     if (threadIdx.x == 0) {
         a.inv_norm[mi] = (float)(1.0 / (sqrt(total) + (double)a.eps));
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(kThreads) muon_normalize_kernel(const Normaliz
     const int block = (int)(a.backward ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
     const int mi = warp_find(a.tile_begin, a.n, block);
     const DevMat &d = a.mats[mi];
-    const int t = block - __ldg(a.tile_begin + mi);
+    const int t = block - ld_table(a.tile_begin + mi);
     const bool tall = d.rows > d.cols, packets = d.cols % kPacket == 0;
     pdl_wait();
     const float s = a.inv_norm[mi];
@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(kThreads) muon_apply_kernel(const ApplyArgs a)
     const int mi = warp_find(a.ch.begin, a.ch.n, block);
     const DevMat &d = a.mats[mi];
     const int64_t n = d.rows * d.cols;
-    const int64_t lo = (int64_t)(block - __ldg(a.ch.begin + mi)) * a.ch.elems;
+    const int64_t lo = (int64_t)(block - ld_table(a.ch.begin + mi)) * a.ch.elems;
     const int64_t hi = lo + a.ch.elems < n ? lo + a.ch.elems : n;
     pdl_wait();
     const ApplyScalars sc = a.dev != nullptr ? *a.dev : ApplyScalars{a.lr, a.lr_wd, a.ef_now};
@@ -454,7 +454,7 @@ __global__ void __launch_bounds__(kThreads) muon_predict_kernel(const ApplyArgs 
     if (d.sync || d.ef == nullptr)
         return;
     const int64_t n = d.rows * d.cols;
-    const int64_t lo = (int64_t)((int)blockIdx.x - __ldg(a.ch.begin + mi)) * a.ch.elems;
+    const int64_t lo = (int64_t)((int)blockIdx.x - ld_table(a.ch.begin + mi)) * a.ch.elems;
     const int64_t hi = lo + a.ch.elems < n ? lo + a.ch.elems : n;
     const ApplyScalars sc = a.dev != nullptr ? *a.dev : ApplyScalars{a.lr, a.lr_wd, a.ef_now};
     const float lr_r = sc.lr * d.r_scale, lr_wd = sc.lr_wd * d.wd_lr_scale;

@@ -113,7 +113,7 @@ __device__ __forceinline__ void finish(double total, double max_norm, double *no
 // chunk. Deterministic for a given numel.
 template <class GT>
 __global__ void __launch_bounds__(kThreads)
-noalloc_sqnorm_kernel(const GT *__restrict__ grad, int64_t numel, int64_t chunk,
+noalloc_sqnorm_kernel(const GT *grad, int64_t numel, int64_t chunk,
                       double max_norm, double *partials, double *norm_out, float *clip_out)
 {
     __shared__ double red[kThreads / 32];

@@ -39,7 +39,7 @@ template <> struct RawPacket<__nv_bfloat16> {
     uint4 q;
     __device__ __forceinline__ void load(const __nv_bfloat16 *p)
     {
-        q = __ldcs(reinterpret_cast<const uint4 *>(p));
+        q = ld_packet(p);
     }
     __device__ __forceinline__ float sqsum() const
     {
@@ -112,7 +112,7 @@ __device__ __forceinline__ double ordered_sum(const double *partials, int n, dou
 {
     double acc = 0.0;
     for (int i = threadIdx.x; i < n; i += NT)
-        acc += __ldcg(partials + i);
+        acc += ld_partial(partials + i);
     return block_sum<NT>(acc, red);
 }
 

@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(kStepThreads) fused_step_kernel(const StepArgs
         float *__restrict__ nn = d.n;
         float *__restrict__ gpv = d.grad_prev;
         float *__restrict__ ef = d.ef;
-        const GT *__restrict__ grad = static_cast<const GT *>(d.grad);
+        const GT *grad = static_cast<const GT *>(d.grad);
         const float wd_lr = (d.flags & kFlagWd) ? sc.lr_wd : 0.0f;
         // A DPO_SYNC tensor takes the standard update with no stash and no
         // correction even while the run is delayed.
