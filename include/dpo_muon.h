@@ -175,6 +175,21 @@ int dpo_muon_clear_status(dpo_muon_ctx *ctx, void *cuda_stream);
 int dpo_muon_test_stall(dpo_muon_ctx *ctx, int launches);
 
 /*
+ * Test hook for the choice of GEMM forms: the output tiles of one
+ * Newton-Schulz product (0: X X^T, 1: c A A + b A, 2: B X + a X) as
+ * dpo_muon_init lays them out for these n matrices (only rows and cols are
+ * read) where `pairs` CTA pairs and `ctas` single CTAs of the kernel are
+ * resident; both 0: what the current device holds. counts receives the tiles
+ * taken by single CTAs and by CTA pairs, and of the pairs' tiles those with a
+ * half in the padding and those drained by four epilogue warps. Returns
+ * DPO_OK, DPO_EINVAL (also for a set of more than DPO_MUON_TEST_MAX_TILES
+ * pair tiles, whose workspace would take terabytes) or DPO_ECUDA.
+ */
+#define DPO_MUON_TEST_MAX_TILES (1 << 24)
+int dpo_muon_test_tiles(const dpo_matrix *mats, int n, int pairs, int ctas, int product,
+                        int64_t *counts);
+
+/*
  * Capturable mode for CUDA graphs, as dpo_set_capturable (dpo.h): the step
  * counters move to device memory, and each dpo_muon_step forms its update's
  * lr, lr wd and EF start (t >= 2) on the device, so a step captured in a

@@ -647,6 +647,155 @@ struct Group {
     CUtensorMap st_x[2], st_xt, st_a, st_b;   // 32 x 32 store boxes of X, X^T, A, B
 };
 
+// The matrices by their wide orientation r x w (r <= w); empty ones in no group.
+std::vector<Group> group_shapes(const dpo_matrix *mats, int n)
+{
+    std::vector<Group> groups;
+    std::map<std::pair<int64_t, int64_t>, int> gidx;
+    for (int i = 0; i < n; ++i) {
+        const dpo_matrix &m = mats[i];
+        if (m.rows * m.cols == 0)
+            continue;
+        const int64_t r = std::min(m.rows, m.cols), w = std::max(m.rows, m.cols);
+        auto key = std::make_pair(r, w);
+        if (!gidx.count(key)) {
+            gidx[key] = (int)groups.size();
+            Group g;
+            g.r = r;
+            g.w = w;
+            g.R = pad_up(r);
+            g.W = pad_up(w);
+            groups.push_back(g);
+        }
+        Group &g = groups[gidx[key]];
+        g.mats.push_back(i);
+        g.has_tall = g.has_tall || m.rows > m.cols;
+    }
+    return groups;
+}
+
+// CTA pairs and single CTAs the GEMM kernels keep resident at once.
+cudaError_t gemm_residency(int sms, int *pairs, int *ctas)
+{
+    *pairs = *ctas = 1 << 30;
+    cudaError_t e = cudaSuccess;
+    for (int form = 0; form < 6 && e == cudaSuccess; ++form) {
+        const int cg = form < 2 ? 1 : 2, ew = form < 4 ? 8 : 4;
+        const void *fn = (const void *)gemm_kernel(form & 1, cg, ew);
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 dpo::gemm::kSmemBytes);
+        int n_res = 0;
+        if (e == cudaSuccess) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(2 * std::max(1, sms / 2));
+            cfg.blockDim = dim3(dpo::gemm::gemm_threads(ew));
+            cfg.dynamicSmemBytes = dpo::gemm::kSmemBytes;
+            e = cudaOccupancyMaxActiveClusters(&n_res, fn, &cfg);
+        }
+        int &have = cg == 2 ? *pairs : *ctas;
+        have = std::min(have, n_res);
+    }
+    return e;
+}
+
+// Tiles of the three products, all by CTA pairs.
+int64_t pair_tiles(const std::vector<Group> &groups)
+{
+    int64_t tiles = 0;
+    for (const Group &g : groups) {
+        const int64_t m = g.R / dpo::gemm::TM, n = g.W / dpo::gemm::TN;
+        tiles += (int64_t)g.mats.size() * (m * (m + 1) + m * n);
+    }
+    return tiles;
+}
+
+// The GEMM launches of a Newton-Schulz step: launch sets and their tiles.
+struct GemmPlan {
+    bool grouped = false;
+    std::vector<LaunchSet> sets;
+    std::vector<int4> tiles;
+};
+
+GemmPlan plan_gemms(const dpo_matrix *mats, const std::vector<Group> &groups, int pairs, int ctas)
+{
+    GemmPlan plan;
+    // When some shape group's launches are short (at most 16 rounds of tiles
+    // over the CTA pairs), each product of a Newton-Schulz step covers all
+    // shape groups in one launch: one group's tiles fill the pairs another
+    // leaves idle, and a step takes 3 launches instead of 3 per group (GPT-2:
+    // every group short; the Llama-1B set's 512 x 2048 group: 20.08 -> 19.80
+    // ms of GEMMs per step on GB300). Sets whose groups are all long keep one
+    // group per launch and run the groups' chains one after another (7B set:
+    // 0.3% slower grouped; two chains at once on two streams mixed their
+    // operands in L2, 336 -> 410 ms per step).
+    int64_t min_tiles = INT64_MAX;
+    for (const Group &g : groups)
+        min_tiles = std::min<int64_t>(min_tiles, (int64_t)g.mats.size() *
+                                                     (g.R / dpo::gemm::TM) * (g.W / dpo::gemm::TN));
+    plan.grouped = groups.size() > 1 && min_tiles <= 16 * (int64_t)std::max(1, pairs);
+    // Launch sets and their tile tables. A launch takes its groups with more K
+    // blocks first: the pairs take tiles round-robin, so the longest tiles go
+    // out first and the short ones fill the last round.
+    std::vector<int4> &tiles = plan.tiles;
+    const int per_set = plan.grouped ? dpo::gemm::kMaxGroups : 1;
+    for (int g0 = 0; g0 < (int)groups.size(); g0 += per_set) {
+        LaunchSet ls;
+        ls.n = std::min(per_set, (int)groups.size() - g0);
+        for (int q = 0; q < ls.n; ++q)
+            ls.group[q] = g0 + q;
+        for (int prod = 0; prod < 3; ++prod) {
+            auto &p = ls.prod[prod];
+            auto k_of = [&](int q) {
+                const Group &g = groups[ls.group[q]];
+                return prod == 0 ? g.w : g.r;
+            };
+            for (int q = 0; q < ls.n; ++q)
+                p.order[q] = q;
+            std::stable_sort(p.order, p.order + ls.n, [&](int x, int y) { return k_of(x) > k_of(y); });
+            std::vector<int4> list[2];   // by single CTAs, by pairs
+            std::vector<int> k_blocks[2];
+            for (int cg = 1; cg <= 2; ++cg) {
+                const int side = dpo::gemm::kTile(cg);
+                for (int q = 0; q < ls.n; ++q) {
+                    const Group &g = groups[ls.group[p.order[q]]];
+                    const int64_t rows = g.r, cols = prod == 2 ? g.w : g.r;
+                    const dpo::gemm::TileGrid tg{(int)((rows + side - 1) / side),
+                                                 (int)((cols + side - 1) / side),
+                                                 (int)g.mats.size(), prod != 2, side};
+                    if (cg == 1 && tg.count() + (int64_t)list[0].size() > kFewRounds * ctas) {
+                        list[0].clear();
+                        break;
+                    }
+                    const int kb = (int)((k_of(p.order[q]) + dpo::gemm::BK - 1) / dpo::gemm::BK);
+                    tg.walk([&](int b, int m0, int n0) {
+                        int flags = 0;
+                        if (cg == 2)
+                            flags = (rows <= m0 + side / 2 ? dpo::gemm::kTileHalfM : 0) |
+                                    (cols <= n0 + side / 2 ? dpo::gemm::kTileHalfN : 0);
+                        const dpo_matrix &m = mats[g.mats[(size_t)b]];
+                        if (m.rows > m.cols)
+                            flags |= dpo::gemm::kTileTall;
+                        list[cg - 1].push_back(make_int4(q | flags, b, m0, n0));
+                        k_blocks[cg - 1].push_back(kb);
+                    });
+                }
+            }
+            p.cg = !list[0].empty() && launch_clocks(k_blocks[0], ctas, 1) <
+                                           launch_clocks(k_blocks[1], pairs, 2)
+                       ? 1
+                       : 2;
+            p.first = (int64_t)tiles.size();
+            p.tiles = (int)list[p.cg - 1].size();
+            if (p.cg == 2 && p.tiles > kLongRounds * pairs &&
+                *std::min_element(k_blocks[1].begin(), k_blocks[1].end()) >= kLongBlocks)
+                p.ew = 4;
+            tiles.insert(tiles.end(), list[p.cg - 1].begin(), list[p.cg - 1].end());
+        }
+        plan.sets.push_back(ls);
+    }
+    return plan;
+}
+
 }  // namespace
 
 struct dpo_muon_ctx {
@@ -835,26 +984,11 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
     cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
 
-    // Group the matrices by their wide orientation r x w (r <= w).
-    std::map<std::pair<int64_t, int64_t>, int> gidx;
+    c->groups = group_shapes(mats, n);
     for (int i = 0; i < n; ++i) {
-        const dpo_matrix &m = mats[i];
-        const int64_t ne = m.rows * m.cols;
-        c->total_elems += ne;
-        if (ne == 0)
-            continue;
-        const int64_t r = std::min(m.rows, m.cols), w = std::max(m.rows, m.cols);
-        auto key = std::make_pair(r, w);
-        if (!gidx.count(key)) {
-            gidx[key] = (int)c->groups.size();
-            Group g;
-            g.r = r;
-            g.w = w;
-            g.R = pad_up(r);
-            g.W = pad_up(w);
-            c->groups.push_back(g);
-        }
-        c->groups[gidx[key]].mats.push_back(i);
+        const int64_t r = std::min(mats[i].rows, mats[i].cols);
+        const int64_t w = std::max(mats[i].rows, mats[i].cols);
+        c->total_elems += r * w;
         // unique entries of the symmetric products X X^T (r (r + 1) / 2, each
         // w multiply-adds) and A A (r (r + 1) / 2, r each), all of B X
         c->flops += (double)hp->ns_steps * ((double)r * (r + 1) * w + (double)r * (r + 1) * r +
@@ -885,109 +1019,18 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
 
     // Workspace: per group X twice, X^T (the output of tall matrices), A, B (bf16).
     int64_t ws = 0;
-    for (Group &g : c->groups) {
+    for (const Group &g : c->groups) {
         const int64_t nb = (int64_t)g.mats.size();
         ws += nb * (g.R * g.W * 3 + g.R * g.R * 2) * 2;
-        for (int mi : g.mats)
-            g.has_tall = g.has_tall || mats[mi].rows > mats[mi].cols;
     }
     c->ws_bytes = ws;
-    // CTA pairs and single CTAs the GEMM kernels keep resident at once (a
-    // failure is reported after the allocations, where the launches it stops
-    // would come).
-    c->gemm_pairs = c->gemm_ctas = 1 << 30;
-    cudaError_t e_gemm = cudaSuccess;
-    for (int form = 0; form < 6 && e_gemm == cudaSuccess; ++form) {
-        const int cg = form < 2 ? 1 : 2, ew = form < 4 ? 8 : 4;
-        const void *fn = (const void *)gemm_kernel(form & 1, cg, ew);
-        e_gemm = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      dpo::gemm::kSmemBytes);
-        int n_res = 0;
-        if (e_gemm == cudaSuccess) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(2 * std::max(1, c->sms / 2));
-            cfg.blockDim = dim3(dpo::gemm::gemm_threads(ew));
-            cfg.dynamicSmemBytes = dpo::gemm::kSmemBytes;
-            e_gemm = cudaOccupancyMaxActiveClusters(&n_res, fn, &cfg);
-        }
-        int &have = cg == 2 ? c->gemm_pairs : c->gemm_ctas;
-        have = std::min(have, n_res);
-    }
-    // When some shape group's launches are short (at most 16 rounds of tiles
-    // over the CTA pairs), each product of a Newton-Schulz step covers all
-    // shape groups in one launch: one group's tiles fill the pairs another
-    // leaves idle, and a step takes 3 launches instead of 3 per group (GPT-2:
-    // every group short; the Llama-1B set's 512 x 2048 group: 20.08 -> 19.80
-    // ms of GEMMs per step on GB300). Sets whose groups are all long keep one
-    // group per launch and run the groups' chains one after another (7B set:
-    // 0.3% slower grouped; two chains at once on two streams mixed their
-    // operands in L2, 336 -> 410 ms per step).
-    int64_t min_tiles = INT64_MAX;
-    for (const Group &g : c->groups)
-        min_tiles = std::min<int64_t>(min_tiles, (int64_t)g.mats.size() *
-                                                     (g.R / dpo::gemm::TM) * (g.W / dpo::gemm::TN));
-    c->grouped = c->groups.size() > 1 && min_tiles <= 16 * (int64_t)std::max(1, c->gemm_pairs);
-    // Launch sets and their tile tables. A launch takes its groups with more K
-    // blocks first: the pairs take tiles round-robin, so the longest tiles go
-    // out first and the short ones fill the last round.
-    std::vector<int4> tiles;
-    const int per_set = c->grouped ? dpo::gemm::kMaxGroups : 1;
-    for (int g0 = 0; g0 < (int)c->groups.size(); g0 += per_set) {
-        LaunchSet ls;
-        ls.n = std::min(per_set, (int)c->groups.size() - g0);
-        for (int q = 0; q < ls.n; ++q)
-            ls.group[q] = g0 + q;
-        for (int prod = 0; prod < 3; ++prod) {
-            auto &p = ls.prod[prod];
-            auto k_of = [&](int q) {
-                const Group &g = c->groups[ls.group[q]];
-                return prod == 0 ? g.w : g.r;
-            };
-            for (int q = 0; q < ls.n; ++q)
-                p.order[q] = q;
-            std::stable_sort(p.order, p.order + ls.n, [&](int x, int y) { return k_of(x) > k_of(y); });
-            std::vector<int4> list[2];   // by single CTAs, by pairs
-            std::vector<int> k_blocks[2];
-            for (int cg = 1; cg <= 2; ++cg) {
-                const int side = dpo::gemm::kTile(cg);
-                for (int q = 0; q < ls.n; ++q) {
-                    const Group &g = c->groups[ls.group[p.order[q]]];
-                    const int64_t rows = g.r, cols = prod == 2 ? g.w : g.r;
-                    const dpo::gemm::TileGrid tg{(int)((rows + side - 1) / side),
-                                                 (int)((cols + side - 1) / side),
-                                                 (int)g.mats.size(), prod != 2, side};
-                    if (cg == 1 && tg.count() + (int64_t)list[0].size() >
-                                       kFewRounds * c->gemm_ctas) {
-                        list[0].clear();
-                        break;
-                    }
-                    const int kb = (int)((k_of(p.order[q]) + dpo::gemm::BK - 1) / dpo::gemm::BK);
-                    tg.walk([&](int b, int m0, int n0) {
-                        int flags = 0;
-                        if (cg == 2)
-                            flags = (rows <= m0 + side / 2 ? dpo::gemm::kTileHalfM : 0) |
-                                    (cols <= n0 + side / 2 ? dpo::gemm::kTileHalfN : 0);
-                        const dpo_matrix &m = mats[g.mats[(size_t)b]];
-                        if (m.rows > m.cols)
-                            flags |= dpo::gemm::kTileTall;
-                        list[cg - 1].push_back(make_int4(q | flags, b, m0, n0));
-                        k_blocks[cg - 1].push_back(kb);
-                    });
-                }
-            }
-            p.cg = !list[0].empty() && launch_clocks(k_blocks[0], c->gemm_ctas, 1) <
-                                           launch_clocks(k_blocks[1], c->gemm_pairs, 2)
-                       ? 1
-                       : 2;
-            p.first = (int64_t)tiles.size();
-            p.tiles = (int)list[p.cg - 1].size();
-            if (p.cg == 2 && p.tiles > kLongRounds * c->gemm_pairs &&
-                *std::min_element(k_blocks[1].begin(), k_blocks[1].end()) >= kLongBlocks)
-                p.ew = 4;
-            tiles.insert(tiles.end(), list[p.cg - 1].begin(), list[p.cg - 1].end());
-        }
-        c->sets.push_back(ls);
-    }
+    // (a failure is reported after the allocations, where the launches it stops
+    // would come)
+    const cudaError_t e_gemm = gemm_residency(c->sms, &c->gemm_pairs, &c->gemm_ctas);
+    const GemmPlan plan = plan_gemms(mats, c->groups, c->gemm_pairs, c->gemm_ctas);
+    c->grouped = plan.grouped;
+    c->sets = plan.sets;
+    const std::vector<int4> &tiles = plan.tiles;
     // Norm-pass table (the elementwise path's gradient-norm kernel).
     int64_t total_pkts = 0;
     std::vector<int64_t> pkt_begin(n + 1, 0);
@@ -1569,6 +1612,37 @@ extern "C" int dpo_muon_test_stall(dpo_muon_ctx *c, int launches)
     if (launches < 0)
         return mfail(c, DPO_EINVAL, "launches must be >= 0");
     c->stall_launches = launches;
+    return DPO_OK;
+}
+
+extern "C" int dpo_muon_test_tiles(const dpo_matrix *mats, int n, int pairs, int ctas, int product,
+                                   int64_t *counts)
+{
+    if (n < 0 || (n > 0 && mats == nullptr) || pairs < 0 || ctas < 0 || (pairs > 0) != (ctas > 0) ||
+        product < 0 || product > 2 || counts == nullptr)
+        return DPO_EINVAL;
+    for (int i = 0; i < n; ++i)
+        if (mats[i].rows < 0 || mats[i].cols < 0)
+            return DPO_EINVAL;
+    if (pairs == 0) {
+        int device = 0, sms = 0;
+        if (cudaGetDevice(&device) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+            gemm_residency(sms, &pairs, &ctas) != cudaSuccess || pairs < 1 || ctas < 1)
+            return DPO_ECUDA;
+    }
+    const std::vector<Group> groups = group_shapes(mats, n);
+    if (pair_tiles(groups) > DPO_MUON_TEST_MAX_TILES)
+        return DPO_EINVAL;
+    const GemmPlan plan = plan_gemms(mats, groups, pairs, ctas);
+    std::fill(counts, counts + 4, 0);
+    for (const LaunchSet &ls : plan.sets) {
+        const auto &p = ls.prod[product];
+        counts[p.cg - 1] += p.tiles;
+        counts[3] += p.ew == 4 ? p.tiles : 0;
+        for (int64_t t = p.first; t < p.first + p.tiles; ++t)
+            counts[2] += (plan.tiles[t].x & (dpo::gemm::kTileHalfM | dpo::gemm::kTileHalfN)) != 0;
+    }
     return DPO_OK;
 }
 

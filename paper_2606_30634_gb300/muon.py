@@ -39,7 +39,7 @@ EXPORTS = ("dpo_muon_init", "dpo_muon_step", "dpo_muon_set_delay", "dpo_muon_las
            "dpo_muon_set_timing", "dpo_muon_get_gemm_time",
            "dpo_muon_workspace_bytes", "dpo_muon_last_error", "dpo_muon_destroy",
            "dpo_muon_grad_sqnorm", "dpo_muon_set_clip_source", "dpo_muon_clear_status",
-           "dpo_muon_test_stall", "dpo_muon_get_phase_start", "dpo_muon_set_phase_start",
+           "dpo_muon_test_stall", "dpo_muon_test_tiles", "dpo_muon_get_phase_start", "dpo_muon_set_phase_start",
            "dpo_muon_set_capturable")
 
 _typed = False
@@ -72,6 +72,8 @@ def lib() -> ctypes.CDLL:
             "dpo_muon_set_clip_source": (I, [P, P]),
             "dpo_muon_clear_status": (I, [P, P]),
             "dpo_muon_test_stall": (I, [P, I]),
+            "dpo_muon_test_tiles": (I, [ctypes.POINTER(dpo_matrix), I, I, I, I,
+                                        ctypes.POINTER(ctypes.c_int64)]),
             "dpo_muon_get_phase_start": (I, [P, ctypes.POINTER(ctypes.c_int64)]),
             "dpo_muon_set_phase_start": (I, [P, ctypes.c_int64]),
             "dpo_muon_set_capturable": (I, [P, I, P, P]),
@@ -95,6 +97,18 @@ def hparams(momentum=0.95, weight_decay=0.1, ef_lambda=1.0, max_grad_norm=0.0,
     return dpo_muon_hparams(momentum, weight_decay, ef_lambda, max_grad_norm, coeffs[0],
                             coeffs[1], coeffs[2], ns_eps, rms_scale, ns_steps, delay,
                             correction)
+
+
+def gemm_tiles(shapes: Sequence[Tuple[int, int]], product: int, pairs: int = 0,
+               ctas: int = 0) -> Tuple[int, int, int, int]:
+    """dpo_muon_test_tiles: (tiles of single CTAs, of CTA pairs, of these with a
+    padded half, of these drained by four epilogue warps)."""
+    mats = (dpo_matrix * max(1, len(shapes)))(*[dpo_matrix(rows=r, cols=c) for r, c in shapes])
+    counts = (ctypes.c_int64 * 4)()
+    rc = lib().dpo_muon_test_tiles(mats, len(shapes), pairs, ctas, product, counts)
+    if rc != DPO_OK:
+        raise DpoError(rc, "dpo_muon_test_tiles")
+    return tuple(counts)
 
 
 class DelayedMuon:

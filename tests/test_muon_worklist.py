@@ -3,7 +3,9 @@ oracle (Alg. 2), at the sizes where the split can go wrong: matrices one
 element short of, at and past one round of a CTA (2048), widths that are no
 whole packets (a packet of the update then spans two or more rows), a last
 partial packet, empty matrices at either end, and more matrices than one warp
-searches at a time (32)."""
+searches at a time (32); and of the GEMMs' tiles, by every form a launch takes.
+Which form a set takes is asked of the library (muon.gemm_tiles), so that a
+change of the rule cannot leave a test without its subject."""
 from __future__ import annotations
 
 import numpy as np
@@ -55,51 +57,89 @@ def test_more_shape_groups_than_one_launch_takes(cuda_device):
         p.close()
 
 
-# sizes on either side of a tile's half (128) and whole (256), in both dimensions
-HALVES = [(127, 129), (128, 128), (129, 384), (256, 385), (257, 640), (384, 257), (385, 513),
-          (512, 641), (640, 640)]
+# sizes on either side of a single CTA's tile (128) and of a pair's (256), in
+# both dimensions; few enough tiles that single CTAs take them
+EDGE_TILES = [(127, 129), (128, 128), (129, 384), (256, 385), (257, 640), (384, 257),
+              (385, 513), (512, 641), (640, 640)]
+# wide, tall and square matrices whose sizes, rounded up to 128, are odd
+# multiples of it in one dimension, the other or both, and enough of them that
+# CTA pairs take all three products
+HALVES = [(640, 640), (600, 1100), (1100, 600), (897, 1152), (1152, 897)] * 6
+
+
+def near_oracle(p, steps, calls=1):
+    """Each matrix's Newton-Schulz output, call by call, at the normwise and
+    differing-elements bars of its steps."""
+    for _ in range(calls):
+        p.step()
+        for i, (g, r) in enumerate(zip(*p.o_pairs())):
+            assert np.linalg.norm(g - r) <= NS_BARS[steps][0] * np.linalg.norm(r), (i, p.shapes[i])
+            assert np.mean(g != r) <= NS_BARS[steps][1], (i, p.shapes[i])
+
+
+@pytest.mark.parametrize("steps", [1, 2])
+def test_tiles_of_single_ctas_at_their_edges(cuda_device, steps):
+    for product in range(3):
+        single, pair, _, _ = muon.gemm_tiles(EDGE_TILES, product)
+        assert single > 0 and pair == 0
+    p = Pair(EDGE_TILES, cuda_device, ns_steps=steps)
+    try:
+        near_oracle(p, steps, calls=2)
+    finally:
+        p.close()
 
 
 @pytest.mark.parametrize("steps", [1, 2])
 def test_tiles_half_in_the_padding(cuda_device, steps):
-    """Matrices whose last tiles are half padding, wide and tall, over two
-    calls (the second reads scratch that the first left): normwise and
-    differing elements of each Newton-Schulz output at the bars of its steps."""
+    """CTA pairs skip the padded half of a tile in all three products, wide and
+    tall (which store X^T alone), over two calls (the second reads scratch that
+    the first left)."""
+    for product in range(3):
+        single, pair, half, four = muon.gemm_tiles(HALVES, product)
+        assert single == 0 and 0 < half < pair and four == 0
     p = Pair(HALVES, cuda_device, ns_steps=steps)
     try:
-        for _ in range(2):
-            p.step()
-            for shape, g, r in zip(HALVES, *p.o_pairs()):
-                assert np.linalg.norm(g - r) <= NS_BARS[steps][0] * np.linalg.norm(r), shape
-                assert np.mean(g != r) <= NS_BARS[steps][1], shape
+        near_oracle(p, steps, calls=2)
     finally:
         p.close()
 
 
-@pytest.mark.parametrize("shape,copies", [((128, 128), 1), ((129, 257), 1), ((256, 768), 2),
-                                          ((640, 300), 3), ((512, 2048), 40), ((768, 768), 60)])
-def test_tiles_by_single_ctas_and_by_pairs(cuda_device, shape, copies):
+# with the form of each product: by single CTAs (1) or by pairs (2)
+FORMS = [((128, 128), 1, (1, 1, 1)), ((129, 257), 1, (1, 1, 1)), ((256, 768), 2, (1, 1, 1)),
+         ((640, 300), 3, (1, 1, 1)), ((512, 2048), 40, (1, 1, 2)), ((768, 768), 60, (2, 2, 2))]
+
+
+@pytest.mark.parametrize("shape,copies,forms", FORMS)
+def test_tiles_by_single_ctas_and_by_pairs(cuda_device, shape, copies, forms):
     """One shape from one tile to several rounds of them: the small sets' GEMMs
     go to single CTAs (128 x 128 tiles), the large sets' to CTA pairs. Two
-    Newton-Schulz steps, so each product reads what the other forms wrote; the
-    first, a middle and the last matrix at the bars of two steps."""
+    Newton-Schulz steps, so each product reads what the other forms wrote."""
+    for product, form in enumerate(forms):
+        tiles = muon.gemm_tiles([shape] * copies, product)
+        assert tiles[form - 1] > 0 and tiles[2 - form] == 0, (product, tiles)
     p = Pair([shape] * copies, cuda_device, ns_steps=2)
     try:
-        p.step()
-        got, ref = p.o_pairs()
-        for i in {0, copies // 2, copies - 1}:
-            assert np.linalg.norm(got[i] - ref[i]) <= NS_BARS[2][0] * np.linalg.norm(ref[i]), i
-            assert np.mean(got[i] != ref[i]) <= NS_BARS[2][1], i
+        near_oracle(p, 2)
     finally:
         p.close()
+
+
+LONG_K = [(4098, 4100), (4100, 4098)]
 
 
 def test_four_epilogue_warps_match_eight(cuda_device):
     """K of 4098 and 4100 (33 blocks, the last nearly empty): a wide and a tall
     matrix together are 578 pair tiles in B X + a X, which four epilogue warps
     drain; each alone is 289, which eight do. The same tiles either way, so the
-    same bits."""
-    shapes = [(4098, 4100), (4100, 4098)]
+    same bits. The symmetric products of one alone go to single CTAs, which
+    compute the same elements from the same K blocks."""
+    shapes = LONG_K
+    for product in range(3):
+        _, pair, half, four = muon.gemm_tiles(shapes, product)
+        assert four == pair > 0 and half > 0
+        for shape in shapes:
+            assert muon.gemm_tiles([shape], product)[3] == 0
+    assert muon.gemm_tiles(shapes[:1], 2)[:3] == (0, 289, 33)
     gen = torch.Generator().manual_seed(7)
     grads = [torch.randn(s, generator=gen) for s in shapes]
 
