@@ -613,7 +613,8 @@ int64_t launch_clocks(const std::vector<int> &k_blocks, int slots, int cg)
 // GB300, eight against four warps, whole step: the 7B set 332.0 -> 323.8 ms, a 7B
 // layer 10370 -> 10180 us, six 2048-wide layers 8107 -> 8063 us. Shorter K needs
 // the eight (kEpiWarps), and so does a launch whose last tile is much of it.
-constexpr int kLongBlocks = 16, kLongRounds = 4;
+constexpr int kLongBlocks = 16;
+constexpr int64_t kLongRounds = 4;   // 64 bits: a failed residency query leaves 2^30 pairs
 
 // Rounds of single-CTA tiles above which a launch goes to the pairs unweighed.
 constexpr int64_t kFewRounds = 4;
