@@ -614,7 +614,7 @@ int64_t launch_clocks(const std::vector<int> &k_blocks, int slots, int cg)
 // layer 10370 -> 10180 us, six 2048-wide layers 8107 -> 8063 us. Shorter K needs
 // the eight (kEpiWarps), and so does a launch whose last tile is much of it.
 constexpr int kLongBlocks = 16;
-constexpr int64_t kLongRounds = 4;   // 64 bits: a failed residency query leaves 2^30 pairs
+constexpr int64_t kLongRounds = 4;
 
 // Rounds of single-CTA tiles above which a launch goes to the pairs unweighed.
 constexpr int64_t kFewRounds = 4;
@@ -1028,10 +1028,14 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
     // (a failure is reported after the allocations, where the launches it stops
     // would come)
     const cudaError_t e_gemm = gemm_residency(c->sms, &c->gemm_pairs, &c->gemm_ctas);
-    const GemmPlan plan = plan_gemms(mats, c->groups, c->gemm_pairs, c->gemm_ctas);
-    c->grouped = plan.grouped;
-    c->sets = plan.sets;
-    const std::vector<int4> &tiles = plan.tiles;
+    // Room for the GEMM tile table, at most: a launch goes to single CTAs with up
+    // to kFewRounds rounds of them, four in the place of a pair's. The table is
+    // made once the workspace is there: that of a set far past the device would
+    // take the host's memory before the allocation could fail.
+    const int64_t by_pairs = pair_tiles(c->groups);
+    const int64_t max_tiles =
+        by_pairs + 3 * std::min<int64_t>(by_pairs, (int64_t)c->groups.size() * kFewRounds *
+                                                       (e_gemm == cudaSuccess ? c->gemm_ctas : 0));
     // Norm-pass table (the elementwise path's gradient-norm kernel).
     int64_t total_pkts = 0;
     std::vector<int64_t> pkt_begin(n + 1, 0);
@@ -1082,7 +1086,7 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
     const int64_t o_asc = off;
     off += al(sizeof(dpo::muon::ApplyScalars));
     const int64_t o_tiles = off;
-    off += al((int64_t)(sizeof(int4) * std::max<size_t>(1, tiles.size())));
+    off += al((int64_t)sizeof(int4) * std::max<int64_t>(1, max_tiles));
 
     cudaError_t e = dpo::device_alloc(&c->dev_block, (size_t)off);
     if (e != cudaSuccess) {
@@ -1097,6 +1101,18 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
                          (long long)ws);
         }
     }
+    if (e_gemm != cudaSuccess || c->gemm_pairs < 1 || c->gemm_ctas < 1) {
+        free_ctx(c);
+        return e_gemm != cudaSuccess ? mcuda(nullptr, e_gemm, "GEMM launch configuration")
+                                     : mfail(nullptr, DPO_ECUDA, "GEMM kernel cannot be resident");
+    }
+    const GemmPlan plan = plan_gemms(mats, c->groups, c->gemm_pairs, c->gemm_ctas);
+    if ((int64_t)plan.tiles.size() > max_tiles) {
+        free_ctx(c);
+        return mfail(nullptr, DPO_ECUDA, "GEMM tile table larger than its room");
+    }
+    c->grouped = plan.grouped;
+    c->sets = plan.sets;
     char *blk = static_cast<char *>(c->dev_block);
     c->d_mats = reinterpret_cast<DevMat *>(blk + o_mats);
     c->d_partials = reinterpret_cast<double *>(blk + o_part);
@@ -1204,7 +1220,7 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
     MUON_COPY(c->d_norm_table, ntab.data(), sizeof(dpo::DevTensor) * n);
     MUON_COPY(c->d_pkt_begin, pkt_begin.data(), sizeof(int64_t) * (n + 1));
     MUON_COPY(c->d_chunk_begin, chunk_begin.data(), sizeof(int) * (n + 1));
-    MUON_COPY(c->d_tiles, tiles.data(), sizeof(int4) * tiles.size());
+    MUON_COPY(c->d_tiles, plan.tiles.data(), sizeof(int4) * plan.tiles.size());
     MUON_COPY(c->d_tile_begin, tile_begin.data(), sizeof(int) * (n + 1));
 #undef MUON_COPY
     e = cudaMemsetAsync(c->d_err, 0, sizeof(unsigned int), s);
@@ -1217,11 +1233,6 @@ extern "C" int dpo_muon_init(dpo_muon_ctx **out, const dpo_matrix *mats, int n,
     if (e != cudaSuccess) {
         free_ctx(c);
         return mcuda(nullptr, e, "workspace clear");
-    }
-    if (e_gemm != cudaSuccess || c->gemm_pairs < 1 || c->gemm_ctas < 1) {
-        free_ctx(c);
-        return e_gemm != cudaSuccess ? mcuda(nullptr, e_gemm, "GEMM launch configuration")
-                                     : mfail(nullptr, DPO_ECUDA, "GEMM kernel cannot be resident");
     }
     if (init_mode == DPO_INIT_FRESH) {
         const int rc = launch_init(c, s, 1, 1);

@@ -7,6 +7,8 @@ import ctypes
 import glob
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -113,6 +115,30 @@ def test_muon_init_rejects(case, code):
         hp = muon.hparams(correction=3)
     rc, out, msg = _muon_init(mats, hp, **kw)
     assert rc == code and out is None and msg
+
+
+_TOO_LARGE = """
+import ctypes, resource, sys
+sys.path.insert(0, sys.argv[1])
+resource.setrlimit(resource.RLIMIT_AS, (16 << 30, 16 << 30))
+from paper_2606_30634_gb300 import dpo, muon
+b, n = 1 << 40, 1 << 26
+m = muon.dpo_matrix(b, b, b, b, None, b, n, n, dpo.DPO_WD_ON)
+out, hp = ctypes.c_void_p(123), muon.hparams()
+rc = muon.lib().dpo_muon_init(ctypes.byref(out), ctypes.byref(m), 1, dpo.DPO_BF16, dpo.DPO_BF16,
+                              ctypes.byref(hp), dpo.DPO_INIT_RESUME, None)
+print(rc, out.value)
+"""
+
+
+def test_muon_init_of_a_set_past_any_device():
+    """A matrix whose workspace no device holds (10^11 tiles): DPO_ENOMEM from
+    the first allocation, with no host table of the tiles before it (in a process
+    of its own, whose memory is limited)."""
+    r = subprocess.run([sys.executable, "-c", _TOO_LARGE, ROOT], capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0, r.stderr[-500:]
+    assert r.stdout.split() == [str(dpo.DPO_ENOMEM), "None"]
 
 
 # ---- host-side validation (returns before any CUDA call) -----------------

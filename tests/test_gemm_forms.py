@@ -50,7 +50,7 @@ def test_bad_arguments(kw):
 
 @pytest.mark.parametrize("pairs", [1 << 28, (1 << 29) - 1, 1 << 29, 1 << 30])
 def test_rounds_of_a_failed_residency_query(pairs):
-    """dpo_muon_init plans with 2^30 pairs when the residency query fails: fewer
-    than one round of tiles, so not the four warps of long launches."""
+    """Fewer than one round of tiles, however many pairs: not the four warps of long
+    launches. (A residency query that fails leaves 2^30.)"""
     for product in range(3):
         assert tiles(LONG_K, product, pairs)[3] == 0
