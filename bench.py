@@ -382,6 +382,20 @@ def build_step(args, w, world, rank, dev, stream, sync=None, **kw):
     return opt, sum(b - a for _, a, b in pieces), step
 
 
+def step_launches(clipped: bool, shared_norm: bool) -> int:
+    """Kernels of one element-wise step: the fused step; with clipping the norm
+    pass, whose partial sums the fused step adds up; with a norm over several
+    ranks also the kernel of dpo_grad_sqnorm that adds them to the scalar."""
+    return 1 + (0 if not clipped else 2 if shared_norm else 1)
+
+
+def muon_launches(correction: int) -> int:
+    """Kernels of one dpo_muon_step without clipping beside its GEMMs: momentum,
+    normalisation and update over all matrices, and with the updated-state
+    prediction momentum, normalisation and prediction once more."""
+    return 6 if correction == 2 else 3
+
+
 def run_gpu(args, w, world, rank, local):
     import torch
 
@@ -401,12 +415,9 @@ def run_gpu(args, w, world, rank, local):
     torch.cuda.synchronize(dev)
     step_bytes, norm_bytes = dpo.dpo_algorithmic_bytes(opt.ctx)
     step_ctas, norm_ctas, threads = dpo.dpo_launch_config(opt.ctx)
-    launches_per_step = 2 if w.max_grad_norm > 0 else 1
-    if sharded(args, world) and w.max_grad_norm > 0:
-        # the norm pass runs through dpo_grad_sqnorm (into the all-reduced
-        # scalar), then one thread forms the coefficient: 3 launches
+    launches_per_step = step_launches(w.max_grad_norm > 0, sharded(args, world))
+    if sharded(args, world) and w.max_grad_norm > 0:   # dpo_grad_sqnorm's pass over the gradients
         norm_bytes = (2 if w.grad_dtype == W.BF16 else 4) * n_local
-        launches_per_step = 3
 
     for _ in range(args.warmup):
         one_step()
@@ -615,13 +626,8 @@ def run_muon(args, w, world, rank, local):
                              W.GRAD_SIGMA)
     torch.cuda.synchronize(dev)
     flops = mo.flops()
-    n_groups = len({(min(r, c), max(r, c)) for r, c in shapes})
-    # AdamW's fused step; momentum, norm, apply; one normalisation per shape
-    # group (the GEMM launches are counted by the library: shape groups may
-    # share them)
-    other_launches_per_step = 1 + 3 + n_groups
-    if corr == 2:   # the updated-state prediction: momentum, norm, predict, normalisations
-        other_launches_per_step += 3 + n_groups
+    # beside the GEMM launches, which the library counts: shape groups may share them
+    other_launches_per_step = step_launches(False, False) + muon_launches(corr)
 
     mo.set_timing(True)
     for _ in range(args.warmup):

@@ -59,9 +59,9 @@ def test_muon_line_with_graph_replay(capsys):
                           "--warmup", "3", "--no-cpu-baseline", "--no-library-ns", "--graph"])
     r = line["roofline"]
     assert r["bound"] == "tensor" and r["unit"] == "TFLOP/s" and 0.1 < r["frac"] < 1.3
-    # AdamW's step, momentum, norm, apply, one normalisation per shape group
-    # (3) and 15 GEMM launches (the three groups share each product's launch)
-    assert line["gpu_launches"] == 3 * (1 + 3 + 3 + 15)
+    # AdamW's step; momentum, normalisation and update; 15 GEMM launches (the
+    # three shape groups share each product's launch)
+    assert line["gpu_launches"] == 3 * (1 + 3 + 15)
     assert line["graph"]["ms_per_step"] > 0
 
 
@@ -72,3 +72,60 @@ def test_muon_entry_of_the_default_line():
     assert entry["value"] > 0 and entry["steps"] == 2
     g = entry["gemm"]
     assert g["bound"] == "tensor" and 0.1 < g["frac"] < 1.3 and g["gemm_ms_per_step"] > 0
+
+
+def _own_kernels(fn):
+    """The library's kernels that one fn() launches, by the profiler's record (the
+    first session of a process may miss what starts with it: none seen, once more)."""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    own = ("fused_step_kernel", "grad_sqnorm_kernel", "norm_finish_kernel", "ns_gemm_kernel",
+           "muon_")
+    for _ in range(3):
+        torch.cuda.synchronize()
+        with profile(activities=[ProfilerActivity.CPU, ProfilerActivity.CUDA]) as prof:
+            fn()
+            torch.cuda.synchronize()
+        n = sum(e.count for e in prof.key_averages() if any(k in e.key for k in own))
+        if n:
+            return n
+    return 0
+
+
+@pytest.mark.parametrize("correction", [0, 1, 2])
+def test_muon_launch_count_is_what_runs(cuda_device, correction):
+    """Three shape groups, so a launch per group would show."""
+    from paper_2606_30634_gb300 import muon
+    m = muon.DelayedMuon([(256, 512), (300, 200), (64, 64)], ef=True, correction=correction,
+                         device=cuda_device)
+    try:
+        m.set_timing(True)
+
+        def step():
+            m.gemm_time()   # starts a new count
+            m.step()
+        step()
+        n = _own_kernels(step)
+        assert n == bench.muon_launches(correction) + m.gemm_time()[1]
+    finally:
+        m.close()
+
+
+@pytest.mark.parametrize("clipped,shared", [(False, False), (True, False), (True, True)])
+def test_step_launch_count_is_what_runs(cuda_device, clipped, shared):
+    import torch
+    from paper_2606_30634_gb300 import dpo
+    opt = dpo.DelayedAdamW([5000, 70], max_grad_norm=0.5 if clipped else 0.0, device=cuda_device)
+    try:
+        acc = torch.zeros(1, dtype=torch.float64, device=cuda_device)
+        if shared:
+            opt.set_clip_source(acc)
+
+        def step():
+            if shared:
+                dpo.global_sqnorm([opt], acc)
+            opt.step()
+        step()
+        assert _own_kernels(step) == bench.step_launches(clipped, shared)
+    finally:
+        opt.close()

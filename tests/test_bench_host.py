@@ -188,3 +188,11 @@ def test_ns_gemm_traffic_follows_the_newton_schulz_steps():
     assert bench.committed_traffic(bench.ns_gemm_tag("llama-7B", 3), "dram_bytes_per_step") is None
     assert bench.committed_traffic(bench.ns_gemm_tag("llama-1B", 5), "dram_bytes_per_step") is None
     assert bench.ns_gemm_tag("llama-7B", 5) == "ns_gemm:llama-7B:ns5"
+
+
+def test_launch_counts():
+    """Kernels per step beside the Newton-Schulz GEMMs; the GPU tests hold these
+    to what the profiler sees."""
+    assert [bench.step_launches(c, s) for c, s in
+            ((False, False), (False, True), (True, False), (True, True))] == [1, 1, 2, 3]
+    assert [bench.muon_launches(c) for c in (0, 1, 2)] == [3, 3, 6]
