@@ -484,8 +484,6 @@ def run_secondary(args, dev, world):
     torch.cuda.synchronize(dev)
     step_bytes, norm_bytes = dpo.dpo_algorithmic_bytes(opt.ctx)
     _, norm_ctas, _ = dpo.dpo_launch_config(opt.ctx)
-    if sharded(args, world):   # the norm pass runs outside dpo_step (dpo_grad_sqnorm)
-        norm_bytes = 2 * n_local
     for _ in range(args.warmup):
         one_step()
     torch.cuda.synchronize(dev)
@@ -511,8 +509,23 @@ def run_secondary(args, dev, world):
     norm_ms = max_over_ranks(norm_ms / calls, world, dev)
     fused_ms = max_over_ranks(fused_ms / calls, world, dev)
     peak, peak_kind = measured_hbm_peak()
-    n = n_local
+    units = w.n_params if sharded(args, world) else w.n_params * world
+    return {"workload": f"{w.name}: {w.n_params} params in {len(w.tensors)} tensors, EF "
+                        f"(lambda=1), global-norm clip at {w.max_grad_norm}, fp32 stash, "
+                        "one-step delay",
+            "value": units * K / (total_ms / 1e3), "unit": UNIT, "steps": K,
+            "params_per_rank": n_local,
+            "ms_per_step": total_ms / K, "grad_norm": gnorm, "clip_coef": coef,
+            "peak": peak, "peak_kind": peak_kind, "norm_ctas": norm_ctas,
+            **clipped_kernel_entries(w.name, n_local, step_bytes, norm_bytes, norm_ms, fused_ms,
+                                     peak, sharded(args, world))}
 
+
+def clipped_kernel_entries(name, n, step_bytes, norm_bytes, norm_ms, fused_ms, peak, shared_norm):
+    """Per-kernel figures of the clipped step from the events inside dpo_step,
+    over n parameters. With a norm shared over ranks no kernel lies between the
+    first two events (dpo_grad_sqnorm and the all-reduce come before the call),
+    so the norm pass and the pair have none."""
     def kern(bytes_, ms, tag):
         t = committed_traffic(tag)
         return {"avg_launch_ms": ms, "algorithmic_bytes_per_launch": bytes_,
@@ -520,24 +533,16 @@ def run_secondary(args, dev, world):
                 "frac": bytes_ / (ms / 1e3) / 1e9 / peak,
                 "traffic": None if t is None else t * n, "traffic_tag": tag}
 
-    pair_ms = norm_ms + fused_ms
-    units = w.n_params if sharded(args, world) else w.n_params * world
-    return {"workload": f"{w.name}: {w.n_params} params in {len(w.tensors)} tensors, EF "
-                        f"(lambda=1), global-norm clip at {w.max_grad_norm}, fp32 stash, "
-                        "one-step delay",
-            "value": units * K / (total_ms / 1e3), "unit": UNIT, "steps": K,
-            "params_per_rank": n_local,
-            "norm_timing": ("grad_sqnorm_kernel inside dpo_step" if not sharded(args, world)
-                            else "dpo_grad_sqnorm + fp64 all-reduce outside dpo_step; "
-                                 "grad_sqnorm_kernel's entry times only the coefficient kernel"),
-            "ms_per_step": total_ms / K, "grad_norm": gnorm, "clip_coef": coef,
-            "peak": peak, "peak_kind": peak_kind, "norm_ctas": norm_ctas,
-            "grad_sqnorm_kernel": kern(norm_bytes, norm_ms, f"grad_sqnorm:{w.name}"),
-            "fused_step_kernel": kern(step_bytes, fused_ms, f"fused_step:{w.name}:ef"),
-            "pair": {"bytes_per_param": (norm_bytes + step_bytes) / n,
-                     "achieved_gbs": (norm_bytes + step_bytes) / (pair_ms / 1e3) / 1e9,
-                     "frac": (norm_bytes + step_bytes) / (pair_ms / 1e3) / 1e9 / peak,
-                     "kernel_ms": pair_ms}}
+    fused = kern(step_bytes, fused_ms, f"fused_step:{name}:ef")
+    if shared_norm:
+        return {"norm_timing": "none: dpo_grad_sqnorm + fp64 all-reduce outside dpo_step",
+                "grad_sqnorm_kernel": None, "fused_step_kernel": fused, "pair": None}
+    both, pair_ms = norm_bytes + step_bytes, norm_ms + fused_ms
+    return {"norm_timing": "grad_sqnorm_kernel inside dpo_step",
+            "grad_sqnorm_kernel": kern(norm_bytes, norm_ms, f"grad_sqnorm:{name}"),
+            "fused_step_kernel": fused,
+            "pair": {"bytes_per_param": both / n, "achieved_gbs": both / (pair_ms / 1e3) / 1e9,
+                     "frac": both / (pair_ms / 1e3) / 1e9 / peak, "kernel_ms": pair_ms}}
 
 
 def run_muon_secondary(args, w, world, rank, local):

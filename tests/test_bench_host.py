@@ -196,3 +196,17 @@ def test_launch_counts():
     assert [bench.step_launches(c, s) for c, s in
             ((False, False), (False, True), (True, False), (True, True))] == [1, 1, 2, 3]
     assert [bench.muon_launches(c) for c in (0, 1, 2)] == [3, 3, 6]
+
+
+def test_clipped_entries_time_only_what_runs_between_the_events():
+    """One rank: both kernels and the pair. A norm over ranks runs before the
+    call, so its (empty) event interval gives no rate and no bytes."""
+    kw = dict(n=1000, step_bytes=40_000, norm_bytes=2000, norm_ms=0.5, fused_ms=2.0, peak=1e-2)
+    one = bench.clipped_kernel_entries("none", shared_norm=False, **kw)
+    assert one["grad_sqnorm_kernel"]["achieved_gbs"] == pytest.approx(2000 / 5e-4 / 1e9)
+    assert one["pair"]["bytes_per_param"] == 42 and one["pair"]["kernel_ms"] == 2.5
+    # dpo_algorithmic_bytes counts no norm pass with a clip source
+    many = bench.clipped_kernel_entries("none", shared_norm=True,
+                                        **dict(kw, norm_bytes=0, norm_ms=0.0))
+    assert many["grad_sqnorm_kernel"] is None and many["pair"] is None
+    assert many["fused_step_kernel"] == one["fused_step_kernel"]
