@@ -255,14 +255,19 @@ int set_step_grid(dpo_ctx *c)
     // A set of at most ten CTAs' packets per SM gets one packet per thread: in
     // two or three rounds the last is nearly empty, and a thread passes over
     // many small tensors from one round to the next. GB300: a flat 2^20 fp32
-    // step 6.05 -> 5.55 us, a clipped one on 1M elements in 120 tensors 19.7 ->
-    // 15.9; at 20 CTAs' packets NAdam on 3M in 150 tensors loses (30.8 ->
-    // 32.6). A clipped step on few tensors keeps to one wave of CTAs, since
-    // each of them adds the norm's partial sums up first (1M in 2 tensors: 11.2
-    // -> 12.7 with a second wave).
+    // step 6.05 -> 5.55 us; at 20 CTAs' packets NAdam on 3M in 150 tensors loses
+    // (30.8 -> 32.6). A clipped step of more than one wave pays for it, since
+    // every CTA adds the norm's partial sums up first, and takes it only where a
+    // thread would pass over many tensors: from 64 that hold elements (empty
+    // ones are never passed over). Clipped AdamW EF, all bf16, persistent / one
+    // packet per thread, 2^20 elements in 1 tensor and 31 empty ones 11.3 / 13.3
+    // us, in 32 equal ones 12.9 / 13.4, in 64 14.8 / 13.8, in 120 19.1 / 15.2;
+    // 1.4M in 32 15.5 / 17.0, in 64 16.8 / 17.2.
     const int64_t sms = std::max(1, c->sms), width = dpo::kStepThreads;
     const bool one_wave = c->total_pkts <= sms * std::max(1, per_sm) * width;
-    if (c->total_pkts <= 10 * sms * width && (one_wave || !c->clip || c->n >= 32))
+    const auto filled = std::count_if(c->table.begin(), c->table.end(),
+                                      [](const dpo_tensor &t) { return t.numel > 0; });
+    if (c->total_pkts <= 10 * sms * width && (one_wave || !c->clip || filled >= 64))
         c->step_grid = (int)std::max<int64_t>(1, (c->total_pkts + width - 1) / width);
     else
         c->step_grid = grid_of(c, std::min(per_sm, want), dpo::kStepThreads);

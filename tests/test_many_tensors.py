@@ -39,3 +39,20 @@ def test_clipped_step_over_many_tensors(cuda_device, n):
         assert dpo.dpo_get_flags(opt.ctx)[1] == pytest.approx(norm, rel=1e-6)
     finally:
         opt.close()
+
+
+def test_empty_tensors_do_not_change_the_launch(cuda_device):
+    """A clipped step of more than one wave is launched by how many tensors a
+    thread passes over; empty ones are not passed over."""
+    def ctas(numels):
+        opt = dpo.DelayedAdamW(numels, ef=True, stash_dtype=dpo.DPO_BF16, max_grad_norm=1.0,
+                               device=cuda_device)
+        try:
+            return dpo.dpo_launch_config(opt.ctx)[0]
+        finally:
+            opt.close()
+
+    n = 1 << 20
+    one = ctas([n])
+    assert ctas([n] + [0] * 200) == one == ctas([n // 63] * 63)
+    assert ctas([n // 64] * 64) == n // 8 // 128 > one
