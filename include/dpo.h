@@ -341,19 +341,21 @@ int dpo_algorithmic_bytes(const dpo_ctx *ctx, int64_t *step_bytes,
                           int64_t *norm_bytes);
 
 /* Launch geometry chosen at init: CTAs of the fused step and of the norm
- * pass (both persistent: a multiple of the SM count for sets large enough to
- * fill the GPU) and threads per CTA of the fused step. */
+ * pass (a multiple of the SM count, persistent, for sets large enough; one
+ * packet per thread of the step, fewer than the most per thread of the norm
+ * pass, for small ones) and threads per CTA of the fused step. */
 int dpo_launch_config(const dpo_ctx *ctx, int *step_ctas, int *norm_ctas,
                       int *threads);
 
 /*
  * Per-kernel timing, for measurement. With timing on, every dpo_step that
  * launches work records three CUDA events on its stream: before the
- * gradient-norm pass (none with a clip source, whose sum the fused step reads), before
- * the fused step, and after it. dpo_get_timing waits for the recorded events,
- * returns the summed milliseconds of the norm interval (*norm_ms, 0 without
- * clipping) and of the fused-step interval (*step_ms) over the *calls timed
- * calls since the last read, and starts a new count. The events' host
+ * gradient-norm pass, before the fused step, and after it. dpo_get_timing
+ * waits for the recorded events, returns the summed milliseconds of the norm
+ * interval (*norm_ms; it holds no kernel without clipping, and none with a
+ * clip source, whose sum the fused step reads) and of the fused-step interval
+ * (*step_ms) over the *calls timed calls since the last read, and starts a new
+ * count. The events' host
  * bookkeeping is not repeated by a CUDA-graph replay: leave timing off while
  * capturing. Returns DPO_OK, DPO_EINVAL or DPO_ECUDA.
  */
@@ -387,9 +389,10 @@ int dpo_get_timing(dpo_ctx *ctx, double *norm_ms, double *step_ms, int64_t *call
  * DPO_NOALLOC_CHUNK_ELEMS elements (smaller chunks for smaller buffers, so
  * they still spread over the SMs); every GPU that loads the library holds
  * it until the process exits. Larger inputs are rejected with DPO_EINVAL.
- * The call allocates nothing: it enqueues one kernel on cuda_stream, or
- * two for a buffer of more than one chunk. The first call on each device looks up the scratch array's
- * device address (cudaGetSymbolAddress) with that device current and keeps
+ * The call allocates nothing: it enqueues one kernel on cuda_stream, or two
+ * for a buffer of more than one chunk. The first call on each device looks up
+ * the scratch array's device address (cudaGetSymbolAddress) with that device
+ * current and keeps
  * it until the process exits, which assumes the device's primary context
  * lives that long (no cudaDeviceReset in between); make that first call
  * before any stream capture. All calls share the scratch array, which keeps

@@ -43,7 +43,8 @@
  * dpo_muon_init, the Newton-Schulz workspace (bf16, for every matrix: two
  * copies of the iterate, its transpose and two Gram-sized matrices, each
  * dimension padded to a multiple of 256) plus a small table and 16 bytes per
- * GEMM tile; no other call allocates or synchronizes the host. All launches go to the stream passed in.
+ * GEMM tile; no other call allocates or synchronizes the host. All launches go
+ * to the stream passed in.
  *
  * Errors. Every call returns DPO_OK (0) or a negative DPO_E* code from
  * dpo.h. dpo_muon_last_error gives the message of the last failing call on a

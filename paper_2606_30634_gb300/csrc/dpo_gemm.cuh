@@ -22,10 +22,11 @@
 //               tcgen05.mma.cta_group::2.kind::f16 (M 256, N 256, K 16) eight
 //               times per stage, reading both CTAs' halves, and commits each
 //               stage and each finished tile to both CTAs;
-//   warps 2-9   epilogue of this CTA's 128 rows: tcgen05.ld 32 lanes x 32
-//               columns at a time, scale, add the addend, round to bf16,
-//               stage the 32 x 32 chunk (and, when asked, its transpose) in
-//               shared memory and write it with a TMA store.
+//   the others  eight warps, or four (EW): epilogue of this CTA's 128 rows:
+//               tcgen05.ld 32 lanes x 32 columns at a time, scale, add the
+//               addend, round to bf16, stage the 32 x 32 chunk (or its
+//               transpose, or both) in shared memory and write it with a
+//               TMA store.
 // Per CTA a stage is 64 KiB for 8.4 MFLOP, a third less than one SM holding
 // a whole 128 x 256 operand pair, so three stages fit and keep the tensor
 // pipe fed across the L2 / DRAM round trip.
@@ -400,10 +401,10 @@ struct GemmGroup {
 // ones 735 -> 702; where no tile has a padded half it costs up to 1 % (two
 // 256x768 matrices 132.0 -> 133.4, GPT-2 1789 -> 1793).
 // Each role of the kernel reads its next entry while it works on the current
-// one. Deriving them from t
-// in the kernel (a search over the groups, four divisions) read the launch's
-// parameters through dependent loads and took every role, the MMA lane among
-// them, some 3,900 cycles per tile: a third of a K = 768 tile's time.
+// one. Deriving them from t in the kernel (a search over the groups, four
+// divisions) read the launch's parameters through dependent loads and took every
+// role, the MMA lane among them, some 3,900 cycles per tile: a third of a
+// K = 768 tile's time.
 constexpr int kTileGroup = 0xff, kTileHalfM = 0x100, kTileHalfN = 0x200, kTileTall = 0x400;
 
 struct GemmLaunch {

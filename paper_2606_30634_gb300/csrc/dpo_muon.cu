@@ -86,8 +86,8 @@ struct Chunks {
     int elems;                // elements per chunk, a multiple of kRound
 };
 
-// Row and column of element e of a matrix with `cols` columns. The 64-bit
-// division is a subroutine of some 70 instructions; most matrices fit 32 bits.
+// Row and column of element e of a matrix with `cols` columns, by the cheaper
+// 32-bit division where the matrix allows it (`small`), as most do.
 __device__ __forceinline__ void row_col(int64_t e, int64_t cols, bool small, int64_t &i, int64_t &j)
 {
     i = small ? (int64_t)((uint32_t)e / (uint32_t)cols) : e / cols;
@@ -610,8 +610,10 @@ int64_t launch_clocks(const std::vector<int> &k_blocks, int slots, int cg)
 // A pair launch of more than kLongRounds rounds of tiles, each of at least
 // kLongBlocks K blocks, is drained by four epilogue warps instead of eight: the
 // next tile's mainloop hides either, and at the power cap the eight cost clocks.
-// GB300, eight against four warps, whole step: the 7B set 332.0 -> 323.8 ms, a 7B
-// layer 10370 -> 10180 us, six 2048-wide layers 8107 -> 8063 us. Shorter K needs
+// GB300, eight against four warps, whole step: the 7B set 332.0 -> 323.8 ms (327.6
+// before the eight came in), a 7B layer 10370 -> 10180 us, six 2048-wide layers
+// 8107 -> 8063 us, each pair from one call (runs of the single layers on another box
+// were 4 % apart: the choice rests on the 7B set). Shorter K needs
 // the eight (kEpiWarps), and so does a launch whose last tile is much of it.
 constexpr int kLongBlocks = 16;
 constexpr int64_t kLongRounds = 4;
