@@ -15,6 +15,7 @@ from oracle.muon import DelayedMuon as OracleMuon, MuonHParams
 from paper_2606_30634_gb300 import dpo, muon, synth
 from parity_util import TOL_RUN, bf16_raw_ulps_above_floor, rel_err
 from test_muon_parity import _flat, close_with_flips, inputs
+from test_muon_worklist import HALVES, LONG_K
 
 pytestmark = pytest.mark.gpu
 
@@ -71,9 +72,8 @@ def test_two_adamw_contexts_on_two_streams(cuda_device):
 
 
 def test_two_muon_contexts_on_two_streams(cuda_device):
-    """Each context's Newton-Schulz GEMMs are persistent launches over every
-    SM; the two streams' launches queue behind one another's CTAs on the
-    device, with no wait between them."""
+    """Each context's Newton-Schulz GEMMs are launches of a few single CTAs,
+    which run beside the other stream's, with no wait between them."""
     sets = [([(256, 768), (768, 256)], 0xC3), ([(300, 700)], 0xD4)]
     lr, ns = 2e-3, 1
     pairs = []
@@ -113,3 +113,37 @@ def test_two_muon_contexts_on_two_streams(cuda_device):
     finally:
         for gpu, _ in pairs:
             gpu.close()
+
+
+def test_two_muon_contexts_of_cta_pairs_on_two_streams(cuda_device):
+    """Both contexts' GEMMs are persistent launches of CTA pairs over every SM,
+    with eight epilogue warps and with four: the streams' launches queue behind
+    one another's CTAs. Every arena equals that of the same steps one context
+    after the other, bit for bit."""
+    sets = [HALVES, LONG_K]
+    for product in range(3):
+        assert muon.gemm_tiles(HALVES, product)[0] == muon.gemm_tiles(HALVES, product)[3] == 0
+        assert muon.gemm_tiles(LONG_K, product)[3] > 0
+
+    def run(at_once):
+        ctxs = []
+        for i, shapes in enumerate(sets):
+            ctxs.append(muon.DelayedMuon(shapes, ef=True, ns_steps=2, device=cuda_device))
+            synth.dev_normal(0xC5 + i, synth.STREAM_GRAD, 1, 0, ctxs[-1].grad, 1e-3)
+        streams = [torch.cuda.Stream(cuda_device) for _ in sets]
+        torch.cuda.synchronize()
+        try:
+            for _ in range(3):
+                for m, s in zip(ctxs, streams):
+                    m.step(stream=s)
+                    if not at_once:
+                        torch.cuda.synchronize()
+            torch.cuda.synchronize()
+            assert all(m.status() == 0 for m in ctxs)
+            return [getattr(m, n).clone() for m in ctxs for n in m.STATE]
+        finally:
+            for m in ctxs:
+                m.close()
+
+    for a, b in zip(run(False), run(True)):
+        assert a.float().abs().sum() > 0 and torch.equal(a, b)

@@ -1,6 +1,8 @@
 """The tensor search of the element-wise kernels against the oracle, at table
 sizes on either side of what one round of it probes (32 entries) and two
-(1024), with runs of empty tensors at both ends and in the middle."""
+(1024), with runs of empty tensors at both ends and in the middle; and the
+launches by set size: one packet per thread or persistent CTAs for the step,
+one to eight packets per thread for the norm pass."""
 from __future__ import annotations
 
 import numpy as np
@@ -56,3 +58,57 @@ def test_empty_tensors_do_not_change_the_launch(cuda_device):
     one = ctas([n])
     assert ctas([n] + [0] * 200) == one == ctas([n // 63] * 63)
     assert ctas([n // 64] * 64) == n // 8 // 128 > one
+
+
+@pytest.mark.parametrize("dtype", [dpo.DPO_F32, dpo.DPO_BF16])
+@pytest.mark.parametrize("pkts", [32768, 32769, 65537, 131073, 262145])
+def test_norm_pass_at_each_width(cuda_device, pkts, dtype):
+    """Sets on either side of where a thread of the norm pass takes 1, 2, 4 and
+    (bf16) 8 packets per round, three ragged tensors: the norm of the clipped step,
+    and dpo_grad_sqnorm's sum, against fp64."""
+    n = 8 * pkts - 3
+    numels = [n // 3, 11, n - n // 3 - 11]
+    opt = dpo.DelayedAdamW(numels, grad_dtype=dtype, max_grad_norm=0.5, device=cuda_device)
+    try:
+        gen = torch.Generator(device=cuda_device).manual_seed(pkts)
+        for i, k in enumerate(numels):
+            opt.grads(i).copy_(torch.randn(k, device=cuda_device, generator=gen).mul_(1e-3))
+        want = sum(float(opt.grads(i).double().square().sum()) for i in range(3))
+        acc = torch.zeros(1, dtype=torch.float64, device=cuda_device)
+        opt.grad_sqnorm(acc)
+        opt.step()
+        # each packet's squares in fp32: 2^-24 each, and as much per Kahan sum
+        assert acc.item() == pytest.approx(want, rel=1e-6)
+        _, norm, clip = dpo.dpo_get_flags(opt.ctx)
+        assert norm == pytest.approx(want ** 0.5, rel=1e-6)
+        assert clip == pytest.approx(0.5 / (want ** 0.5 + 1e-6), rel=1e-6)
+    finally:
+        opt.close()
+
+
+def test_one_packet_per_thread_equals_persistent_ctas(cuda_device):
+    """A flat set at the last size of one packet per thread (ten CTAs' packets per
+    SM) and one element past it, which persistent CTAs take: the shared elements
+    end up the same, bit for bit, over three calls."""
+    sms = torch.cuda.get_device_properties(cuda_device).multi_processor_count
+    n = 10 * sms * 128 * 8
+
+    def run(numel, ctas):
+        gen = torch.Generator(device=cuda_device).manual_seed(3)
+        x0 = torch.randn(n + 1, device=cuda_device, generator=gen)[:numel]
+        opt = dpo.DelayedAdamW([numel], ef=True, stash_dtype=dpo.DPO_BF16, x0=x0,
+                               device=cuda_device)
+        try:
+            assert dpo.dpo_launch_config(opt.ctx)[0] == ctas
+            for _ in range(3):
+                opt.grads(0).copy_(torch.randn(n + 1, device=cuda_device,
+                                               generator=gen)[:numel].mul_(1e-3))
+                opt.step()
+            torch.cuda.synchronize()
+            return [opt.view(a, 0)[:n].clone() for a in (opt.master, opt.m, opt.v, opt.ef,
+                                                         opt.stash, opt.param)]
+        finally:
+            opt.close()
+
+    for a, b in zip(run(n, 10 * sms), run(n + 1, 3 * sms)):
+        assert torch.equal(a, b)

@@ -396,16 +396,24 @@ def test_muon_full_size_shapes(cuda_device):
         gpu.close()
 
 
-def test_gemm_wait_timeout_reports_status(cuda_device):
+# by single CTAs; by CTA pairs with eight epilogue warps, and with four
+STALLED = [([(256, 512), (512, 768)], (1, 0, 0)), ([(768, 768)] * 60, (0, 1, 0)),
+           ([(4098, 4100), (4100, 4098)], (0, 1, 1))]
+
+
+@pytest.mark.parametrize("shapes,form", STALLED, ids=["single", "pairs", "pairs-four-warps"])
+def test_gemm_wait_timeout_reports_status(cuda_device, shapes, form):
     """The failure path of the tensor-core pipeline, without a GPU fault: one
     GEMM launch whose MMA lane waits on a phase nothing completes gives up
     after its one-second limit, every role leaves through its own bounded
     wait, the step returns and the status says which waits gave up
     (4: accumulator hand-off, 2: free stage; not 1 or 8, since every TMA
     stage issued has landed). After clearing, the context and the GPU work
-    on: the next call reports nothing, and a fresh context holds parity."""
+    on: the next call reports nothing, and a fresh context holds parity. The
+    stalled launch is X X^T, by every form of the kernel."""
     import time
-    shapes = [(256, 512), (512, 768)]
+    single, pair, _, four = muon.gemm_tiles(shapes, 0)
+    assert (single > 0, pair > 0, four > 0) == tuple(map(bool, form))
     m = muon.DelayedMuon(shapes, ns_steps=1, device=cuda_device)
     try:
         off = 0
